@@ -1199,15 +1199,15 @@ def overlap_launches(n_arrays):
 
 
 def guarded_check_launches(n_statements, n_vars):
-    """Kernels of one guarded check (two scan passes): the reduce / carry /
-    apply path where the size rule takes it for a trace of that length (5
-    kernels up to 8,192 variables -- warp batches and a two-level carry --
-    else 3) in each pass, or the scan kernel plus, in the second pass, the
-    final-status kernel."""
+    """Kernels of one guarded check: on the reduce / carry / apply path (where
+    the size rule takes it for a trace of that length) up to 65,536 variables
+    sort + reduce, carry, resolve + reduce, carry and apply, above that two
+    passes of three kernels; else two scans, the second with the final-status
+    kernel."""
     import paper_1910_11110_gb300 as amc
     path, n = amc.trace_plan(n_statements, n_vars)
     if path in ("warp_dense", "dense"):
-        return 2 * n
+        return 5 if n_vars <= 65_536 else 2 * n
     return 1 + 2
 
 

@@ -149,8 +149,8 @@ AMC_API int amc_check_trace(const uint8_t* kind_side, const int32_t* var, int64_
  * Returns AMC_E_INVALID for negative sizes. */
 enum { AMC_PATH_SCAN = 0,        /* single-pass scan over linked runs */
        AMC_PATH_SMALL = 1,       /* one CTA: at most 2^16 ops over at most 2,048 variables */
-       AMC_PATH_WARP_DENSE = 2,  /* reduce / carry / apply, warp-sequential chunks */
-       AMC_PATH_DENSE = 3,       /* reduce / carry / apply, sorted tiles */
+       AMC_PATH_WARP_DENSE = 2,  /* reduce / carry / apply, up to 8,192 variables */
+       AMC_PATH_DENSE = 3,       /* reduce / carry / apply, more variables */
        AMC_PATH_PREFIX = 4,      /* a reduce / carry / apply prefix, then the scan */
        AMC_PATH_EPOCHS = 5 };    /* first part sorted by variable, then filtered epochs */
 AMC_API int amc_check_trace_plan(int64_t n_ops, int32_t n_vars, int has_init, int32_t* path, int32_t* launches);
@@ -159,10 +159,10 @@ AMC_API int amc_check_trace_plan(int64_t n_ops, int32_t n_vars, int has_init, in
 AMC_API size_t amc_check_guarded_trace_workspace(int64_t n_ops, int32_t n_vars);
 
 /* amc_check_trace for traces that also contain GT (kind 6), as produced by
- * amc_translate_vectorpu.  Runs two scans: the first yields the status of
- * every EN's variable before the EN with GT read as Noop (guards only read
- * abstract variables, which GT never touches); the second resolves each GT
- * from that status (the condition of Fig. sem-AM is checked on the abstract
+ * amc_translate_vectorpu.  A first pass yields the status of every EN's
+ * variable before the EN with GT read as Noop (guards only read abstract
+ * variables, which GT never touches); a second resolves each GT from that
+ * status (the condition of Fig. sem-AM is checked on the abstract
  * value, Section 3.3) and checks the trace.  Same outputs and errors as
  * amc_check_trace; a GT not followed by an EN of the same side on another
  * variable is reported as AMC_E_INVALID. */

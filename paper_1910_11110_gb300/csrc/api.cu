@@ -315,6 +315,16 @@ int amc_check_guarded_trace(const uint8_t* kind_side, const int32_t* var, int64_
     auto run = [&](int i) {
         ScanLaunch P1 = A;
         if (i == 1) P1.dense = 1;
+        if (scan_guarded_owner(P1)) {
+            // up to 65,536 variables on that path: both passes in one go
+            P1.step = step_status;
+            P1.final_status = final_status;
+            P1.vff = var_first_fault;
+            P1.first_fault = first_fault;
+            P1.pre_mode = 0;
+            P1.profile = 3;
+            return launch_scan_guarded_owner(P1, s);
+        }
         int r = launch_scan_trace(P1, s);
         if (r) return r;
         // pass 2: GT resolved from the pre-status of the EN that follows it

@@ -1,5 +1,7 @@
-// scan_dense.cu -- the trace check for traces over few variables (reduce,
-// carry, apply), where nearly every op stays live.
+// scan_dense.cu -- the reduce / carry / apply trace check: which sizes take it,
+// and its form with a global row per chunk (over more variables than fit a
+// CTA's shared memory, and for the dense start of a long trace).  Up to 65,536
+// variables scan_owner.cu does the work.
 //
 // What it computes is what scan_trace.cu computes: for every op the status of
 // its variable after (or, in the guard pass, before) the op, by applying the
@@ -7,12 +9,13 @@
 // (Section 3.2), so the trace may be cut into chunks whose per-variable
 // compositions are combined afterwards.
 //
-// Over few variables the per-variable lists of the single-pass kernel become
-// long and every tile in flight contends for the same ones.  Here instead:
+// Where nearly every op is live, the per-variable lists of the single-pass
+// kernel become long and every tile in flight contends for the same ones.  Here
+// instead:
 //  1. reduce: CTA c takes chunk c (consecutive 4,096-op tiles) and, tile by
 //     tile, sorts the ops by variable, composes each variable's run and folds
-//     it into a dense per-variable element vector in shared memory; the vector
-//     is written out (one byte per variable and chunk);
+//     it into the chunk's row of transfer functions (a byte per variable, in
+//     global memory);
 //  2. carry: one thread per variable walks the chunks in order, applying the
 //     chunk aggregates to the initial status: the status at every chunk entry
 //     and the final status;
@@ -22,6 +25,7 @@
 #include <cstdlib>
 
 #include "amc_internal.cuh"
+#include "scan_owner.cuh"
 #include "scan_trace.cuh"
 
 namespace amc {
@@ -34,8 +38,8 @@ constexpr int DE = DT / DNT;             // sorted slots per thread
 constexpr int DNW = DNT / 32;
 constexpr int DPOS = 12;                 // log2(DT): position bits of a key
 constexpr int DDIG = 7;                  // radix digit bits
-constexpr int DENSE_MAX_VARS = 16384;    // the dense vector lives in shared memory
-constexpr int DENSE_MAX_CHUNKS = 2048;
+constexpr int DENSE_MAX_VARS = 16384;    // by size up to here
+constexpr int WARP_MAX_VARS = 8192;      // three-kernel carry up to here
 constexpr int64_t DENSE_MIN_OPS = 1 << 10;
 
 __device__ __forceinline__ int dpad(int i) { return i + (i >> 5); }
@@ -77,7 +81,6 @@ struct __align__(16) DenseSmem {
     int scanTmp[DNW + 2];
     uint8_t segF[DNW];
     uint8_t segV[DNW];
-    // followed (dynamic shared memory) by the per-variable vector: n_vars bytes
 };
 
 // One tile: load, decode, sort by variable, segmented scan; then either fold
@@ -337,10 +340,10 @@ __device__ void dense_tile(const DenseParams& p, DenseSmem& S, uint8_t* vec, con
     }
 }
 
-// GV: the per-variable vector is the chunk's own row of aggs (reduce) or entry
-// (apply) in global memory, for variable counts beyond shared memory; the
-// CTA's tiles run in order and only this CTA touches the row.
-template <bool APPLY, bool GV>
+// The per-variable vector is the chunk's own row of aggs (reduce) or entry
+// (apply) in global memory; the CTA's tiles run in order and only this CTA
+// touches the row.
+template <bool APPLY>
 __global__ void __launch_bounds__(DNT) dense_chunk_kernel(const DenseParams p)
 {
     extern __shared__ __align__(16) uint8_t smem[];
@@ -351,25 +354,17 @@ __global__ void __launch_bounds__(DNT) dense_chunk_kernel(const DenseParams p)
     for (int i = tid; i < 256; i += DNT) S.elem_of[i] = p.tab.elem_of[i];
     const int c = blockIdx.x;
     const size_t V = (size_t)p.n_vars;
-    uint8_t* vec;
-    if (GV) {
-        vec = (APPLY ? p.entry : p.aggs) + (size_t)c * V;
-        if (!APPLY) {
-            const uint32_t id4 = p.tab.identity * 0x01010101u;
-            const size_t n16 = (V % 16 == 0) ? V / 16 : 0;
-            for (size_t i = tid; i < n16; i += DNT) reinterpret_cast<uint4*>(vec)[i] = make_uint4(id4, id4, id4, id4);
-            for (size_t v = n16 * 16 + tid; v < V; v += DNT) vec[v] = p.tab.identity;
-        }
-    } else {
-        vec = smem + sizeof(DenseSmem);
-        for (int v = tid; v < p.n_vars; v += DNT) vec[v] = APPLY ? p.entry[(size_t)c * V + v] : p.tab.identity;
+    uint8_t* vec = (APPLY ? p.entry : p.aggs) + (size_t)c * V;
+    if (!APPLY) {
+        const uint32_t id4 = p.tab.identity * 0x01010101u;
+        const size_t n16 = (V % 16 == 0) ? V / 16 : 0;
+        for (size_t i = tid; i < n16; i += DNT) reinterpret_cast<uint4*>(vec)[i] = make_uint4(id4, id4, id4, id4);
+        for (size_t v = n16 * 16 + tid; v < V; v += DNT) vec[v] = p.tab.identity;
     }
     __syncthreads();
     const int t0 = c * p.tiles_per_chunk;
     const int t1 = min(t0 + p.tiles_per_chunk, p.n_tiles);
     for (int t = t0; t < t1; ++t) dense_tile<APPLY>(p, S, vec, t);
-    if (!APPLY && !GV)
-        for (int v = tid; v < p.n_vars; v += DNT) p.aggs[(size_t)c * V + v] = vec[v];
 }
 
 // Thread per four variables (one 32-bit word of every chunk row; rows are
@@ -415,250 +410,6 @@ __global__ void dense_carry_kernel(const DenseParams p)
         e = app[p.aggs[(size_t)c * V + v] * 8 + e];
     }
     if (p.final_status) p.final_status[v] = (uint8_t)e;
-}
-
-// ---------------------------------------------------------------------------
-// Warp-sequential variant for at most 8,192 variables: every warp owns a
-// contiguous sub-chunk (a multiple of 32 ops) and a dense per-variable vector
-// in shared memory, and walks its sub-chunk in batches of 32 consecutive ops.
-// The lanes of a batch that touch the same variable are grouped by match.any;
-// a group's ops are composed in lane (= trace) order from a per-warp staging
-// array, so no sort is needed.  The sub-chunks are the carry's chunks.
-constexpr int WARP_MAX_VARS = 8192;
-constexpr int WARP_CHUNKS_MAX = 8192;
-constexpr int SEG = 64;                 // chunks per carry segment
-
-template <bool APPLY>
-__global__ void __launch_bounds__(256) warp_chunk_kernel(const DenseParams p, const int64_t cs)
-{
-    extern __shared__ __align__(16) uint8_t wsm[];
-    uint8_t* comp = wsm;                                  // [32 * 32]
-    uint8_t* app = comp + MAX_ELEMS * MAX_ELEMS;          // [32 * 8]
-    uint8_t* elem_of = app + MAX_ELEMS * 8;               // [256]
-    uint8_t* mbuf = elem_of + 256;                        // [8 warps][32]
-    uint8_t* vecs = mbuf + 256;                           // [8 warps][n_vars]
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int i = tid; i < MAX_ELEMS * MAX_ELEMS; i += 256) comp[i] = p.tab.comp[i];
-    for (int i = tid; i < MAX_ELEMS * 8; i += 256) app[i] = p.tab.app[i];
-    for (int i = tid; i < 256; i += 256) elem_of[i] = p.tab.elem_of[i];
-    __syncthreads();
-    const int64_t g = (int64_t)blockIdx.x * 8 + warp;
-    if (g >= p.n_chunks) return;                          // no block barrier below
-    const size_t V = (size_t)p.n_vars;
-    const uint32_t ID = p.tab.identity;
-    const uint32_t lt = lanemask_lt();
-    uint8_t* vec = vecs + (size_t)warp * V;
-    uint8_t* mb = mbuf + warp * 32;
-    for (size_t v = lane; v < V; v += 32) vec[v] = APPLY ? p.entry[(size_t)g * V + v] : (uint8_t)ID;
-    __syncwarp();
-    const int64_t lo = g * cs;
-    const int64_t hi = min(lo + cs, p.n_ops);
-    constexpr int UB = 8;                                 // batches whose loads are in flight together
-    for (int64_t b0 = lo; b0 < hi; b0 += 32 * UB) {
-    uint32_t ksb[UB];
-    int32_t vb[UB];
-#pragma unroll
-    for (int u = 0; u < UB; ++u) {
-        const int64_t i = b0 + 32 * u + lane;
-        ksb[u] = i < hi ? (uint32_t)__ldcs(p.kind_side + i) : 0u;
-        vb[u] = i < hi ? __ldcs(p.var + i) : 0;
-    }
-#pragma unroll
-    for (int u = 0; u < UB; ++u) {
-        const int64_t b = b0 + 32 * u;
-        if (b >= hi) break;                               // warp-uniform
-        const int64_t i = b + lane;
-        const bool ok = i < hi;
-        uint32_t ks = ksb[u];
-        int32_t v = vb[u];
-        if (ok) {
-            if ((ks & 0xE0u) || (ks & 15u) > AMC_K_EN) raise_error(p.err, AMC_E_INVALID);
-            if (v < 0 || v >= p.n_vars) {
-                raise_error(p.err, AMC_E_RANGE);
-                v = 0;
-            }
-        }
-        const uint32_t nks_l = __shfl_down_sync(0xffffffffu, ks, 1);
-        const int32_t nv_l = __shfl_down_sync(0xffffffffu, v, 1);
-        uint32_t m = ok ? elem_of[ks] : ID;
-        if (ok && m == ELEM_GT) {
-            // GT must be followed by EN of the same side on another variable
-            uint32_t nks = 0xFF;
-            int32_t nv = v;
-            if (i + 1 < p.n_ops_follow) {
-                const bool in_batch = lane < 31 && i + 1 < hi;
-                nks = in_batch ? nks_l : p.kind_side[i + 1];
-                nv = in_batch ? nv_l : p.var[i + 1];
-            }
-            const bool gt_ok = (nks & 15) == AMC_K_EN && (nks >> 4) == (ks >> 4) && nv != v;
-            if (!gt_ok) raise_error(p.err, AMC_E_INVALID);
-            if (!gt_ok || p.pre_mode) {
-                m = ID;
-            } else if (!p.guard) {
-                raise_error(p.err, AMC_E_INVALID);
-                m = ID;
-            } else {
-                const uint32_t gs = p.guard[i + 1];
-                const int side = ks >> 4;
-                const bool valid = gs != ST_F && (gs & (side == 0 ? 1u : 2u));
-                m = valid ? ID : p.tab.pull_of_side[side];
-            }
-        } else if (m == ELEM_BAD) {
-            m = ID;
-        }
-        mb[lane] = (uint8_t)m;
-        const uint32_t peers = __match_any_sync(0xffffffffu, ok ? (uint32_t)v : 0xFFFFFFFFu);
-        __syncwarp();
-        if constexpr (!APPLY) {
-            if (ok && lane == __ffs(peers) - 1) {             // the group's first lane folds it in
-                uint32_t acc = vec[v];
-                for (uint32_t q = peers; q; q &= q - 1) acc = comp[acc * MAX_ELEMS + mb[__ffs(q) - 1]];
-                vec[v] = (uint8_t)acc;
-            }
-        } else {
-            const uint32_t e = ok ? vec[v] : 0u;                  // the variable's status before the batch
-            __syncwarp();
-            if (ok) {
-                uint32_t acc = ID;
-                for (uint32_t q = peers & lt; q; q &= q - 1) acc = comp[acc * MAX_ELEMS + mb[__ffs(q) - 1]];
-                const uint32_t pre = app[acc * 8 + e];
-                const uint32_t post = app[comp[acc * MAX_ELEMS + m] * 8 + e];
-                p.step[i] = (uint8_t)(p.pre_mode ? pre : post);
-                if (post == ST_F && pre != ST_F) {
-                    atomicMin(reinterpret_cast<uint32_t*>(p.vff) + v, (uint32_t)i);
-                    atomicMin(reinterpret_cast<unsigned long long*>(p.first_fault), (unsigned long long)i);
-                }
-                if (lane == 31 - __clz(peers)) vec[v] = (uint8_t)post;   // the group's last lane
-            }
-        }
-        __syncwarp();
-    }
-    }
-    if constexpr (!APPLY)
-        for (size_t v = lane; v < V; v += 32) p.aggs[(size_t)g * V + v] = vec[v];
-}
-
-// Segmented carry over many chunks: (1) compose each segment's chunk
-// aggregates, (2) carry the initial statuses over the segments, (3) expand
-// every chunk's entry statuses inside its segment.  Thread per (segment,
-// variable); composition is associative, so this equals the serial carry.
-__global__ void seg_reduce_kernel(const DenseParams p, uint8_t* __restrict__ seg_agg, int n_segs)
-{
-    __shared__ uint8_t comp[MAX_ELEMS * MAX_ELEMS];
-    for (int i = threadIdx.x; i < MAX_ELEMS * MAX_ELEMS; i += blockDim.x) comp[i] = p.tab.comp[i];
-    __syncthreads();
-    const size_t V = (size_t)p.n_vars;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (int64_t)n_segs * (int64_t)V) return;
-    const int s = (int)(t / (int64_t)V);
-    const size_t v = (size_t)(t % (int64_t)V);
-    uint32_t acc = p.tab.identity;
-    const int c1 = min((s + 1) * SEG, p.n_chunks);
-    for (int c = s * SEG; c < c1; ++c) acc = comp[acc * MAX_ELEMS + p.aggs[(size_t)c * V + v]];
-    seg_agg[(size_t)s * V + v] = (uint8_t)acc;
-}
-
-__global__ void seg_carry_kernel(const DenseParams p, const uint8_t* __restrict__ seg_agg,
-                                 uint8_t* __restrict__ seg_entry, int n_segs)
-{
-    __shared__ uint8_t app[MAX_ELEMS * 8];
-    for (int i = threadIdx.x; i < MAX_ELEMS * 8; i += blockDim.x) app[i] = p.tab.app[i];
-    __syncthreads();
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= p.n_vars) return;
-    const size_t V = (size_t)p.n_vars;
-    uint32_t e = p.init ? p.init[v] : (uint32_t)AMC_ST_VI;
-    for (int s = 0; s < n_segs; ++s) {
-        seg_entry[(size_t)s * V + v] = (uint8_t)e;
-        e = app[seg_agg[(size_t)s * V + v] * 8 + e];
-    }
-    if (p.final_status) p.final_status[v] = (uint8_t)e;
-}
-
-__global__ void seg_expand_kernel(const DenseParams p, const uint8_t* __restrict__ seg_entry, int n_segs)
-{
-    __shared__ uint8_t app[MAX_ELEMS * 8];
-    for (int i = threadIdx.x; i < MAX_ELEMS * 8; i += blockDim.x) app[i] = p.tab.app[i];
-    __syncthreads();
-    const size_t V = (size_t)p.n_vars;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (int64_t)n_segs * (int64_t)V) return;
-    const int s = (int)(t / (int64_t)V);
-    const size_t v = (size_t)(t % (int64_t)V);
-    uint32_t e = seg_entry[(size_t)s * V + v];
-    const int c1 = min((s + 1) * SEG, p.n_chunks);
-    for (int c = s * SEG; c < c1; ++c) {
-        p.entry[(size_t)c * V + v] = (uint8_t)e;
-        e = app[p.aggs[(size_t)c * V + v] * 8 + e];
-    }
-}
-
-// Warp sub-chunks of a trace: chunk length (a multiple of 32) and count.
-void warp_shape(int64_t n_ops, int64_t& cs, int& n_chunks)
-{
-    int64_t want = (n_ops + 4095) / 4096;                 // at least a tile's worth per warp
-    if (want > WARP_CHUNKS_MAX) want = WARP_CHUNKS_MAX;
-    if (want < 1) want = 1;
-    cs = ((n_ops + want - 1) / want + 31) / 32 * 32;
-    if (cs < 32) cs = 32;
-    n_chunks = (int)((n_ops + cs - 1) / cs);
-}
-
-size_t warp_workspace_bytes(int64_t n_ops, int32_t n_vars)
-{
-    int64_t cs;
-    int n_chunks;
-    warp_shape(n_ops, cs, n_chunks);
-    const int n_segs = (n_chunks + SEG - 1) / SEG;
-    return 2 * align_up((size_t)n_chunks * (size_t)n_vars, 256) + 2 * align_up((size_t)n_segs * (size_t)n_vars, 256);
-}
-
-int launch_warp_dense(const ScanLaunch& L, uint8_t* ws, cudaStream_t s)
-{
-    DenseParams p{};
-    p.kind_side = L.kind_side;
-    p.var = L.var;
-    p.n_ops = L.n_ops;
-    p.n_ops_follow = L.n_ops;
-    p.n_vars = L.n_vars;
-    p.init = L.init;
-    p.step = L.step;
-    p.vff = L.vff;
-    p.first_fault = L.first_fault;
-    p.final_status = L.final_status;
-    p.guard = L.guard;
-    p.pre_mode = L.pre_mode;
-    p.err = L.err;
-    p.tab = host_tables();
-    int64_t cs;
-    warp_shape(L.n_ops, cs, p.n_chunks);
-    const int n_segs = (p.n_chunks + SEG - 1) / SEG;
-    const size_t V = (size_t)L.n_vars;
-    p.aggs = ws;
-    p.entry = ws + align_up((size_t)p.n_chunks * V, 256);
-    uint8_t* seg_agg = p.entry + align_up((size_t)p.n_chunks * V, 256);
-    uint8_t* seg_entry = seg_agg + align_up((size_t)n_segs * V, 256);
-    if (cudaMemsetAsync(L.vff, 0xFF, 4 * V, s) != cudaSuccess) return AMC_E_CUDA;
-    if (cudaMemsetAsync(L.first_fault, 0xFF, 8, s) != cudaSuccess) return AMC_E_CUDA;
-    const size_t smem = MAX_ELEMS * MAX_ELEMS + MAX_ELEMS * 8 + 256 + 256 + 8 * V;
-    if (cudaFuncSetAttribute(warp_chunk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(warp_chunk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess)
-        return AMC_E_CUDA;
-    const unsigned grid = (unsigned)((p.n_chunks + 7) / 8);
-    const unsigned segv = (unsigned)(((int64_t)n_segs * (int64_t)V + 255) / 256);
-    if (L.profile & 1) profile_begin(s);
-    warp_chunk_kernel<false><<<grid, 256, smem, s>>>(p, cs);
-    if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
-    seg_reduce_kernel<<<segv, 256, 0, s>>>(p, seg_agg, n_segs);
-    seg_carry_kernel<<<(unsigned)((V + 255) / 256), 256, 0, s>>>(p, seg_agg, seg_entry, n_segs);
-    seg_expand_kernel<<<segv, 256, 0, s>>>(p, seg_entry, n_segs);
-    if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
-    warp_chunk_kernel<true><<<grid, 256, smem, s>>>(p, cs);
-    if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
-    if (L.profile & 2) profile_end(s);
-    return AMC_OK;
 }
 
 void dense_shape(int64_t n_ops, int max_chunks, int& n_tiles, int& n_chunks, int& tpc)
@@ -722,13 +473,12 @@ int launch_dense_range(const ScanLaunch& L, int max_chunks, int64_t n_follow, ui
     while (kb < 31 && ((int64_t)1 << kb) < (int64_t)L.n_vars) ++kb;
     p.passes = (kb + DDIG - 1) / DDIG;
     p.digit_bits = (kb + p.passes - 1) / p.passes;
-    const bool gv = L.n_vars > DENSE_MAX_VARS;
 
     if (cudaMemsetAsync(L.vff, 0xFF, 4 * (size_t)L.n_vars, s) != cudaSuccess) return AMC_E_CUDA;
     if (cudaMemsetAsync(L.first_fault, 0xFF, 8, s) != cudaSuccess) return AMC_E_CUDA;
-    const size_t smem = sizeof(DenseSmem) + (gv ? 0 : (size_t)L.n_vars);
-    auto kr = gv ? dense_chunk_kernel<false, true> : dense_chunk_kernel<false, false>;
-    auto ka = gv ? dense_chunk_kernel<true, true> : dense_chunk_kernel<true, false>;
+    const size_t smem = sizeof(DenseSmem);
+    auto kr = dense_chunk_kernel<false>;
+    auto ka = dense_chunk_kernel<true>;
     if (cudaFuncSetAttribute(kr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
         cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return AMC_E_CUDA;
@@ -770,12 +520,12 @@ bool scan_dense_eligible(int64_t n_ops, int32_t n_vars)
     return ln >= 15 + 2 * (12 - lv) && n_ops >= DENSE_MIN_OPS;
 }
 
-// The whole trace over more than 16,384 (at most 2^20) variables with global
-// per-chunk rows: where nothing gets stuck (a well-declared program's guarded
-// trace) every op stays live and the single-pass kernel's lists are long and
-// contended.  Taken when the launch forces it (the tuner times it) on traces
-// of at least GV_MIN_OPS ops; chunk count from the row budget (about 2^28
-// row bytes, 256 .. 1,024 chunks).
+// The whole trace over more variables than a CTA's shared memory takes beside
+// a tile (65,536; at most 2^20) with global per-chunk rows: where nothing gets
+// stuck (a well-declared program's guarded trace) every op stays live and the
+// single-pass kernel's lists are long and contended.  Taken when the launch
+// forces it (the tuner times it) on traces of at least GV_MIN_OPS ops; chunk
+// count from the row budget (about 2^28 row bytes, 256 .. 1,024 chunks).
 constexpr int64_t GV_MIN_OPS = (int64_t)1 << 20;
 constexpr int32_t GV_MAX_VARS = 1 << 20;
 
@@ -788,34 +538,26 @@ int gv_chunks(int32_t n_vars)
 bool dense_forced_ok(int64_t n_ops, int32_t n_vars)
 {
     if (n_vars < 1 || n_ops < 1) return false;
-    return n_vars <= DENSE_MAX_VARS || (n_vars <= GV_MAX_VARS && n_ops >= GV_MIN_OPS);
+    return n_vars <= OWN_MAX_VARS || (n_vars <= GV_MAX_VARS && n_ops >= GV_MIN_OPS);
 }
 
 size_t scan_dense_workspace_bytes(int64_t n_ops, int32_t n_vars)
 {
+    if (n_vars < 1 || n_ops < 1) return 0;
     int n_tiles, n_chunks, tpc;
-    if (n_vars > DENSE_MAX_VARS && n_vars <= GV_MAX_VARS && n_ops >= GV_MIN_OPS) {
+    size_t b = 0;
+    if (n_vars <= OWN_MAX_VARS) {
+        b = owner_workspace_bytes(n_ops, n_vars);
+    } else if (n_vars <= GV_MAX_VARS && n_ops >= GV_MIN_OPS) {
         dense_shape(n_ops, gv_chunks(n_vars), n_tiles, n_chunks, tpc);
-        size_t b = 2 * align_up((size_t)n_chunks * (size_t)n_vars, 256);
-        if (const int64_t P = prefix_ops(n_ops, n_vars, false)) {
-            dense_shape(P, PREFIX_CHUNKS, n_tiles, n_chunks, tpc);
-            const size_t pb = 2 * align_up((size_t)n_chunks * (size_t)n_vars, 256) + align_up(4 * (size_t)n_vars, 256) +
-                              256 + align_up((size_t)n_vars, 256) + 256;
-            if (pb > b) b = pb;
-        }
-        return b;
+        b = 2 * align_up((size_t)n_chunks * (size_t)n_vars, 256);
     }
-    if (const int64_t P = prefix_ops(n_ops, n_vars, false)) {   // the larger workspace
+    if (const int64_t P = prefix_ops(n_ops, n_vars, false)) {
         // prefix rows, then the suffix's first faults and the prefix's final statuses
-        dense_shape(P, PREFIX_CHUNKS, n_tiles, n_chunks, tpc);
-        return 2 * align_up((size_t)n_chunks * (size_t)n_vars, 256) + align_up(4 * (size_t)n_vars, 256) + 256 +
-               align_up((size_t)n_vars, 256) + 256;
+        const size_t pb = scan_prefix_workspace_bytes(P, n_vars);
+        if (pb > b) b = pb;
     }
-    if (n_vars < 1 || n_vars > DENSE_MAX_VARS || n_ops < 1) return 0;
-    dense_shape(n_ops, DENSE_MAX_CHUNKS, n_tiles, n_chunks, tpc);
-    const size_t sorted = 2 * align_up((size_t)n_chunks * (size_t)n_vars, 256);
-    const size_t warped = n_vars <= WARP_MAX_VARS ? warp_workspace_bytes(n_ops, n_vars) : 0;
-    return sorted > warped ? sorted : warped;
+    return b;
 }
 
 bool scan_prefix_eligible(int64_t n_ops, int32_t n_vars, bool has_init)
@@ -903,14 +645,33 @@ int launch_scan_prefix(const ScanLaunch& L, uint8_t* ws, cudaStream_t s)
     return AMC_OK;
 }
 
+namespace {
+
+// 256 threads a CTA: above 8,192 variables, or as a test override
+bool owner_wide(int32_t n_vars)
+{
+    const char* e = getenv("AMC_SCAN_DENSE_SORT");
+    return n_vars > WARP_MAX_VARS || (e && e[0] == '1');
+}
+
+}  // namespace
+
 int launch_scan_dense(const ScanLaunch& L, uint8_t* ws, cudaStream_t s)
 {
-    // up to 8,192 variables: warp-sequential batches; else tile sorts (rows
-    // in shared memory up to 16,384 variables, in global memory above)
-    const char* e = getenv("AMC_SCAN_DENSE_SORT");                // test override: the sorted variant
-    if (L.n_vars <= WARP_MAX_VARS && !(e && e[0] == '1')) return launch_warp_dense(L, ws, s);
-    if (L.n_vars > DENSE_MAX_VARS) return launch_dense_range(L, gv_chunks(L.n_vars), L.n_ops, ws, s);
-    return launch_dense_range(L, DENSE_MAX_CHUNKS, L.n_ops, ws, s);
+    if (L.n_vars > OWN_MAX_VARS) return launch_dense_range(L, gv_chunks(L.n_vars), L.n_ops, ws, s);
+    return launch_scan_owner(L, owner_wide(L.n_vars), ws, s);
+}
+
+bool scan_guarded_owner(const ScanLaunch& L)
+{
+    return L.n_vars <= OWN_MAX_VARS && L.dense != 0 &&
+           ((L.dense == 1 && dense_forced_ok(L.n_ops, L.n_vars)) || scan_dense_eligible(L.n_ops, L.n_vars));
+}
+
+int launch_scan_guarded_owner(const ScanLaunch& L, cudaStream_t s)
+{
+    uint8_t* ws = static_cast<uint8_t*>(L.workspace) + scan_workspace_bytes(L.n_ops, L.n_vars, false);
+    return launch_guarded_owner(L, owner_wide(L.n_vars), ws, s);
 }
 
 int launch_merge_faults(int32_t* vff, const int32_t* vff_part, int32_t n_vars, int64_t* ff,

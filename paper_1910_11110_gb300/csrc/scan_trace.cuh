@@ -74,17 +74,23 @@ struct ScanLaunch {
 int scan_tile_size();
 size_t scan_workspace_bytes(int64_t n_ops, int32_t n_vars, bool with_dense = true);
 int launch_scan_trace(const ScanLaunch& L, cudaStream_t s);
-// Traces over at most 16,384 variables take the reduce / carry / apply path of
-// scan_dense.cu by size (or whenever AMC_SCAN_DENSE=1 or the launch forces it;
+// Traces over at most 16,384 variables take the reduce / carry / apply path
+// (scan_owner.cu; scan_dense.cu with rows in global memory above 65,536
+// variables) by size (or whenever AMC_SCAN_DENSE=1 or the launch forces it;
 // never when AMC_SCAN_DENSE=0); its scratch follows the single-pass workspace.
 // By size: at least 1,024 ops and at least 2^(15 + 2 (12 - log2 n_vars)) ops (the crossover with the
 // single-pass scan measured on random traces with the Zipf workload's kind
 // mix: 2^11 ops at 2^14 variables, 2^15 at 2^12, 2^21 at 2^9).
 bool scan_dense_eligible(int64_t n_ops, int32_t n_vars);
 // Whether a launch may force the reduce / carry / apply path on these sizes
-// (at most 16,384 variables; up to 2^20 with global rows from 2^20 ops on).
+// (at most 65,536 variables; up to 2^20 with global rows from 2^20 ops on).
 bool dense_forced_ok(int64_t n_ops, int32_t n_vars);
 size_t scan_dense_workspace_bytes(int64_t n_ops, int32_t n_vars);
+// Whether a guarded check takes that path for both its passes, which then run
+// as one launch sequence (L: the whole check; its workspace is that of
+// scan_workspace_bytes).
+bool scan_guarded_owner(const ScanLaunch& L);
+int launch_scan_guarded_owner(const ScanLaunch& L, cudaStream_t s);
 int launch_scan_dense(const ScanLaunch& L, uint8_t* ws, cudaStream_t s);
 // Traces over more than 16,384 (at most 2^20) variables and of 2^24 ops or
 // more, without initial statuses: the first 2^22 ops take that path with
