@@ -132,14 +132,18 @@ __global__ void ov_zero_kernel(int32_t* __restrict__ cnt, int64_t NL)
     if (a < NL) cnt[a] = 0;
 }
 
-// the pairs after the sort, as ov_idx
-__global__ void ov_copy_kernel(const uint32_t* __restrict__ src, uint32_t* __restrict__ dst, const int64_t* off,
-                               int64_t NL, int64_t cap)
+// the pairs after the sort as list entries: other << 1 | (other's range lies
+// inside the owner's)
+__global__ void ov_copy_kernel(const uint32_t* __restrict__ other, const uint32_t* __restrict__ owner_list,
+                               uint32_t* __restrict__ dst, const OvParams p, int64_t NL)
 {
-    if (off[NL] > cap) return;
-    const int64_t n = off[NL];
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        dst[i] = src[i];
+    if (p.off[NL] > p.cap) return;
+    const int64_t n = p.off[NL];
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t y = other[i], x = owner_list[i] / (uint32_t)p.nb;
+        const int32_t sx = p.start[x], sy = p.start[y];
+        dst[i] = y << 1 | (uint32_t)(sx <= sy && (int64_t)sy + p.len[y] <= (int64_t)sx + p.len[x]);
+    }
 }
 
 struct OvLayout {
@@ -252,8 +256,8 @@ int launch_overlaps(const OverlapBuild& O, cudaStream_t s)
     int dev = 0, n_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    ov_copy_kernel<<<(unsigned)(n_sm > 0 ? 4 * n_sm : 256), 256, 0, s>>>(v2[passes2 & 1], O.ov_idx, O.ov_off, NL,
-                                                                           O.cap);
+    ov_copy_kernel<<<(unsigned)(n_sm > 0 ? 4 * n_sm : 256), 256, 0, s>>>(v2[passes2 & 1], k2[passes2 & 1], O.ov_idx, p,
+                                                                           NL);
     ov_clear_kernel<<<lb, 256, 0, s>>>(O.ov_off, NL, gate);
     return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
 }

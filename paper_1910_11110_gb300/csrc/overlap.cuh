@@ -18,7 +18,7 @@ struct OverlapBuild {
     int64_t bucket_len = 1;               // calls per bucket
     int64_t cap = 0;                      // list entries the output holds; 0: count only
     int64_t* ov_off = nullptr;            // [n_arrays * n_buckets + 1] offsets of list (a, bucket)
-    uint32_t* ov_idx = nullptr;           // [cap] list entries (with cap > 0)
+    uint32_t* ov_idx = nullptr;           // [cap] list entries (with cap > 0): other << 1 | (it lies inside the owner)
     int64_t* n_pairs = nullptr;           // nullable, device: listed pairs (both directions)
     int* err = nullptr;
     void* workspace = nullptr;
