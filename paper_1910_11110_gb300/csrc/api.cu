@@ -631,7 +631,7 @@ int amc_check_batch(const uint8_t* tok_kind_side, const int32_t* tok_payload, co
 size_t amc_check_trace_k_workspace(int64_t n_ops, int32_t n_vars)
 {
     if (n_ops < 0 || n_vars < 0) return 0;
-    return kloc_workspace_bytes(n_ops);
+    return kloc_workspace_bytes(n_ops, n_vars);
 }
 
 int amc_check_trace_k(const uint8_t* op, const int32_t* var, int64_t n_ops, int32_t n_vars, int32_t k,
@@ -643,7 +643,7 @@ int amc_check_trace_k(const uint8_t* op, const int32_t* var, int64_t n_ops, int3
     int rc = check_trace_args(op, var, n_ops, n_vars, step_status, final_status, var_first_fault, first_fault);
     if (rc) return rc;
     if (init_status && init_status == final_status) return AMC_E_INVALID;
-    if (!workspace || !aligned256(workspace) || ws_bytes < kloc_workspace_bytes(n_ops)) return AMC_E_NOMEM;
+    if (!workspace || !aligned256(workspace) || ws_bytes < kloc_workspace_bytes(n_ops, n_vars)) return AMC_E_NOMEM;
     int* err = device_error_word();
     if (!err) return AMC_E_CUDA;
     KlocLaunch L;

@@ -21,7 +21,7 @@ struct KlocLaunch {
     int profile = 0;
 };
 
-size_t kloc_workspace_bytes(int64_t n_ops);
+size_t kloc_workspace_bytes(int64_t n_ops, int32_t n_vars);
 int launch_kloc(const KlocLaunch& L, cudaStream_t s);
 
 }  // namespace amc
