@@ -12,12 +12,19 @@
 //     Y "written" -- with conditions opaque: w maps any state to Y, other ops
 //     keep it, If is the union of its branches' sets and While the closure of
 //     its body.  The obligation holds iff N is not in the set at the end.  The
-//     warp keeps, per tracked location, the bit "N is not in the set" (lane j
-//     owns 64 locations per word): an op sets its bit; at an If the then- and
-//     else-sets come from the same entry, so the bit after it is entry OR
-//     (then AND else); a While may run zero times, so its body adds nothing.
-// The warp walks the body 32 tokens at a time: ops are checked in parallel,
-// structure tokens by the whole warp with a stack of the entry / then bits.
+//     warp keeps, per tracked location, the bit "N is not in the set" (in
+//     shared memory): an op sets its bit; at an If the then- and else-sets come
+//     from the same entry, so the bit after it is entry OR (then AND else); a
+//     While may run zero times, so its body adds nothing.
+// The warp takes the body 32 tokens at a time, the next 32 on their way: all
+// its ops are checked at once (the checks do not depend on the structure), the
+// tracked writes between two structure tokens set their bits with one shared
+// atomic each, and the structure tokens are walked by the whole warp with a
+// stack of the entry / then bits.  What bounds it is the latency of a call's
+// few dependent loads and its instructions, not its bytes (5 per token).
+// 2^20 calls of 38 tokens: 1.57 ms when every write's bit went to its owning
+// lane through 32 shuffles a batch and every structure token reloaded the
+// batch; 0.93 ms here, at 73 % of the issue slots (820 instructions a call).
 #include "amc_internal.cuh"
 #include "wd.cuh"
 
@@ -26,6 +33,7 @@ namespace amc {
 namespace {
 
 constexpr int WD_WARPS = 4;                   // warps per CTA
+constexpr int WD_CLAIM = 8;                   // calls per claim (fewer than 32)
 constexpr int WD_WORDS = 32;                  // tracked words per warp pass: 32 lanes x 64 locations
 
 struct WdParams {
@@ -49,36 +57,39 @@ struct WdParams {
 };
 
 struct WdWarp {
-    int32_t arr[AMC_WD_MAX_DECLS];
-    uint8_t mode[AMC_WD_MAX_DECLS];
+    uint32_t cur[2 * WD_WORDS];                       // the window's bits
+    uint32_t stack[2 * AMC_MAX_DEPTH][2 * WD_WORDS];  // per level: entry bits, then-branch bits
     int64_t base[AMC_WD_MAX_DECLS];       // first tracked bit of a W entry, -1 for R / RW
-    uint64_t stack[2 * AMC_MAX_DEPTH][32];  // per level: entry bits, then-branch bits (per lane word)
     int64_t fend[AMC_MAX_DEPTH];          // END token of each open construct
     int64_t felse[AMC_MAX_DEPTH];         // ELSE token of an open If (-1 for While)
+    int64_t loc0[AMC_WD_MAX_DECLS];       // first location and locations of the array
+    int64_t locs[AMC_WD_MAX_DECLS];
+    int32_t arr[AMC_WD_MAX_DECLS];
+    uint8_t mode[AMC_WD_MAX_DECLS];
 };
 
 __device__ __forceinline__ bool wd_op_kind(uint32_t k) { return k <= AMC_K_NOOP; }
 
-// One call: declarations into shared memory, then one pass over the body per
-// window of WD_WORDS * 64 tracked locations (at least one pass, for the
-// statement checks).
-__device__ void wd_call(const WdParams& p, int64_t c, WdWarp& S)
+// One call (tokens [t0, t1), declarations [m0, m1)): declarations into shared
+// memory, then one pass over the body per window of WD_WORDS * 64 tracked
+// locations (at least one pass, for the statement checks).  I: an integer that
+// holds the body's length; positions below are relative to t0.
+template <typename I>
+__device__ __forceinline__ void wd_call(const WdParams& p, int64_t c, int64_t t0, const I len_t, int64_t m0, const int nd,
+                                        int64_t n_locs, WdWarp& S)
 {
+    constexpr I NONE = sizeof(I) == 4 ? (I)INT32_MAX : (I)INT64_MAX;
     const int lane = threadIdx.x & 31;
-    const int64_t n_locs = p.n_arrays > 0 ? p.arr_loc_off[p.n_arrays] : 0;
-    const int64_t t0 = p.call_tok_off[c], t1 = p.call_tok_off[c + 1];
-    const int64_t m0 = p.call_am_off[c], m1 = p.call_am_off[c + 1];
-    if (t0 < 0 || t1 < t0 || t1 > p.n_tokens || m0 < 0 || m1 < m0 || m1 > p.n_decls ||
-        m1 - m0 > AMC_WD_MAX_DECLS) {
-        if (lane == 0) raise_error(p.err, AMC_E_INVALID);
-        return;
-    }
-    const int nd = (int)(m1 - m0);
+    const uint8_t* const tok = p.tok + t0;
+    const int32_t* const payload = p.payload + t0;
+    // the first tokens, on their way while the declarations are read
+    uint32_t nks = lane < len_t ? tok[lane] : 0xFFu;
+    int32_t npl = lane < len_t ? payload[lane] : 0;
     uint32_t viol = 0;
     // declarations: range, mode, duplicates, tracked bases of the W entries
     int32_t a = -1;
     uint32_t md = 0;
-    int64_t len = 0;
+    int64_t len = 0, loc0 = 0;
     if (lane < nd) {
         a = p.am_array[m0 + lane];
         md = p.am_mode[m0 + lane];
@@ -86,7 +97,8 @@ __device__ void wd_call(const WdParams& p, int64_t c, WdWarp& S)
             raise_error(p.err, AMC_E_RANGE);
             a = -1;
         } else {
-            len = p.arr_loc_off[a + 1] - p.arr_loc_off[a];
+            loc0 = p.arr_loc_off[a];
+            len = p.arr_loc_off[a + 1] - loc0;
         }
         if ((md & 0xE0u) || (md & 15u) < 1 || (md & 15u) > 3) raise_error(p.err, AMC_E_INVALID);
     }
@@ -95,161 +107,194 @@ __device__ void wd_call(const WdParams& p, int64_t c, WdWarp& S)
         if (lane > j && lane < nd && a >= 0 && a == aj) viol |= 16u;     // declared twice
     }
     const bool isw = lane < nd && a >= 0 && (md & 15u) == 2u;
-    int64_t wl = isw ? len : 0;
-    int64_t incl = wl;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int64_t y = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += y;
+    int64_t tracked = 0;
+    for (uint32_t r = __ballot_sync(0xffffffffu, isw); r; r &= r - 1) {  // W entries in order
+        const int j = __ffs(r) - 1;
+        const int64_t n = __shfl_sync(0xffffffffu, (long long)len, j);
+        if (lane == j) S.base[j] = tracked;
+        tracked += n;
     }
-    const int64_t tracked = __shfl_sync(0xffffffffu, incl, 31);
     if (lane < nd) {
         S.arr[lane] = a;
         S.mode[lane] = (uint8_t)md;
-        S.base[lane] = isw ? incl - wl : -1;
+        S.loc0[lane] = loc0;
+        S.locs[lane] = len;
+        if (!isw) S.base[lane] = -1;
     }
     __syncwarp();
-    int64_t bad = INT64_MAX;
+    I bad = NONE;
     int32_t unmet = INT32_MAX;
     bool malformed = false;
-    const int64_t window = (int64_t)WD_WORDS * 64;
+    I range = NONE, stop = NONE;          // first id out of range (per lane); where the body is malformed
+    constexpr int64_t window = (int64_t)WD_WORDS * 64;
+    const bool one_window = tracked <= window;
     for (int64_t w0 = 0; w0 == 0 || w0 < tracked; w0 += window) {
         const bool first_pass = w0 == 0;
-        uint64_t cur = 0;                    // this lane's word: locations w0 + 64 lane + [0, 64)
+        // words in use: lane i owns words i and 32 + i
+        const int words = (int)((min(tracked - w0, window) + 31) / 32);
+        for (int i = lane; i < words; i += 32) S.cur[i] = 0;
+        __syncwarp();
+        if (!first_pass) {
+            nks = lane < len_t ? tok[lane] : 0xFFu;
+            npl = lane < len_t ? payload[lane] : 0;
+        }
         int depth = 0;
-        for (int64_t pos = t0; pos < t1 && !malformed;) {
-            const int64_t q = pos + lane;
-            const bool in = q < t1;
-            const uint32_t ks = in ? p.tok[q] : 0xFFu;
-            const int32_t pl = in ? p.payload[q] : 0;
+        for (I q0 = 0; q0 < len_t && stop == NONE; q0 += 32) {
+            const I q = q0 + lane;
+            const bool in = q < len_t;
+            const uint32_t ks = nks;
+            const int32_t pl = npl;
+            const bool more = len_t - q0 > 32 && q < len_t - 32;
+            nks = more ? tok[q + 32] : 0xFFu;
+            npl = more ? payload[q + 32] : 0;
             const uint32_t k = ks & 15u;
             const bool op = in && !(ks & 0xE0u) && wd_op_kind(k);
-            // the run of op tokens at the head of this batch
-            const uint32_t nonop = __ballot_sync(0xffffffffu, !op);
-            const int cnt = nonop ? __ffs(nonop) - 1 : 32;
-            int64_t bit = -1;
-            if (lane < cnt && k != AMC_K_NOOP) {
+            int bit = -1;
+            if (op && k != AMC_K_NOOP) {
                 if (pl < 0 || pl >= n_locs) {
-                    raise_error(p.err, AMC_E_RANGE);
+                    range = min(range, q);
                 } else if (k == AMC_K_PUSH || k == AMC_K_PULL) {
                     if (first_pass) {
                         viol |= 1u;
-                        bad = min(bad, q - t0);
+                        bad = min(bad, q);
                     }
                 } else {
                     const int32_t own = p.loc_owner[pl];
                     const uint32_t side = (ks >> 4) & 1u;
                     bool ok = false;
                     for (int j = 0; j < nd; ++j) {
-                        if (S.arr[j] != own || ((S.mode[j] >> 4) & 1u) != side) continue;
-                        const uint32_t m = S.mode[j] & 15u;
-                        if (k == AMC_K_W && (m == 2u || m == 3u)) ok = true;
-                        if (k == AMC_K_R && (m == 1u || m == 3u)) ok = true;
-                        if (k == AMC_K_W && m == 2u) bit = S.base[j] + (pl - p.arr_loc_off[own]) - w0;
+                        const uint32_t m = S.mode[j];
+                        if (S.arr[j] != own || ((m >> 4) & 1u) != side) continue;
+                        if (k == AMC_K_W ? (m & 2u) : (m & 1u)) ok = true;      // W, RW; R, RW
+                        if (k == AMC_K_W && (m & 15u) == 2u) {
+                            if (one_window) {
+                                const int b = (int)S.base[j] + (pl - (int)S.loc0[j]);
+                                bit = (uint32_t)b < (uint32_t)window ? b : -1;
+                            } else {
+                                const int64_t b = S.base[j] + (pl - S.loc0[j]) - w0;
+                                bit = b >= 0 && b < window ? (int)b : -1;
+                            }
+                        }
                     }
                     if (!ok && first_pass) {
                         viol |= k == AMC_K_W ? 2u : 4u;
-                        bad = min(bad, q - t0);
+                        bad = min(bad, q);
                     }
                 }
             }
-            // the run's tracked writes set their bits in the owning lanes' words
-            for (int L = 0; L < cnt; ++L) {
-                const int64_t b = __shfl_sync(0xffffffffu, bit, L);
-                if (b >= 0 && b < window && (int)(b >> 6) == lane) cur |= 1ull << (b & 63);
-            }
-            pos += cnt;
-            if (cnt == 32) continue;
-            if (pos >= t1) break;
-            // one structure token, by the whole warp
-            const uint32_t sks = __shfl_sync(0xffffffffu, ks, cnt);
-            const int32_t spl = __shfl_sync(0xffffffffu, pl, cnt);
-            const uint32_t sk = sks & 15u;
-            const int64_t lim = depth ? S.fend[depth - 1] : t1;
-            if (sks & 0xF0u) {                                // structure tokens carry no side
-                malformed = true;
-                break;
-            }
-            if (sk == AMC_T_IF || sk == AMC_T_WHILE) {
-                int64_t e = -1, end = -1;
-                if (spl >= 0) {
-                    if (sk == AMC_T_IF) {
-                        e = pos + 1 + spl;
-                        if (e < lim && p.tok[e] == AMC_T_ELSE && p.payload[e] >= 0) end = e + 1 + p.payload[e];
-                    } else {
+            // the structure tokens in order; the tracked writes before each set their bits
+            int from = 0;
+            // token at x > pos, from the 64 at hand where it is one of them
+            auto tok_at = [&](I x) -> uint32_t {
+                const I d = x - q0;
+                if (d < 64) return __shfl_sync(0xffffffffu, d < 32 ? ks : nks, (int)d & 31);
+                return tok[x];
+            };
+            auto len_at = [&](I x) -> int32_t {
+                const I d = x - q0;
+                if (d < 64) return __shfl_sync(0xffffffffu, d < 32 ? pl : npl, (int)d & 31);
+                return payload[x];
+            };
+            for (uint32_t st = __ballot_sync(0xffffffffu, in && !op);; st &= st - 1) {
+                const int s = st ? __ffs(st) - 1 : 32;
+                if (bit >= 0 && lane >= from && lane < s) atomicOr(&S.cur[bit >> 5], 1u << (bit & 31));
+                __syncwarp();
+                if (!st) break;
+                from = s + 1;
+                const I pos = q0 + s;
+                const uint32_t sks = __shfl_sync(0xffffffffu, ks, s);
+                const int32_t spl = __shfl_sync(0xffffffffu, pl, s);
+                const I lim = depth ? (I)S.fend[depth - 1] : len_t;
+                if (sks == AMC_T_IF || sks == AMC_T_WHILE) {          // structure tokens carry no side
+                    // ends past the enclosing range are malformed: lengths are compared with what is left
+                    I e = -1, end = -1;
+                    const I room = lim - pos - 1;
+                    if (spl >= 0 && spl < room) {
                         end = pos + 1 + spl;
+                        if (sks == AMC_T_IF) {
+                            e = end;
+                            end = -1;
+                            if (tok_at(e) == AMC_T_ELSE) {
+                                const int32_t el = len_at(e);
+                                if (el >= 0 && el < lim - e - 1) end = e + 1 + el;
+                            }
+                        }
                     }
-                }
-                if (end <= pos || end >= lim || p.tok[end] != AMC_T_END || depth >= AMC_MAX_DEPTH) {
-                    malformed = true;
+                    if (end < 0 || tok_at(end) != AMC_T_END || depth >= AMC_MAX_DEPTH) {
+                        stop = pos;
+                        break;
+                    }
+                    for (int i = lane; i < words; i += 32) {          // the branch / body from scratch
+                        S.stack[2 * depth][i] = S.cur[i];             // entry bits
+                        S.cur[i] = 0;
+                    }
+                    if (lane == 0) {
+                        S.fend[depth] = end;
+                        S.felse[depth] = sks == AMC_T_IF ? e : -1;
+                    }
+                    ++depth;
+                } else if (sks == AMC_T_ELSE) {
+                    if (!depth || S.felse[depth - 1] != pos) {
+                        stop = pos;
+                        break;
+                    }
+                    for (int i = lane; i < words; i += 32) {
+                        S.stack[2 * (depth - 1) + 1][i] = S.cur[i];   // then-branch bits
+                        S.cur[i] = 0;
+                    }
+                } else if (sks == AMC_T_END) {
+                    if (!depth || S.fend[depth - 1] != pos) {
+                        stop = pos;
+                        break;
+                    }
+                    --depth;
+                    const bool is_if = S.felse[depth] >= 0;
+                    for (int i = lane; i < words; i += 32)
+                        S.cur[i] = S.stack[2 * depth][i] | (is_if ? S.stack[2 * depth + 1][i] & S.cur[i] : 0u);
+                } else {
+                    stop = pos;                                        // pw / GT / EN, or a byte out of range
                     break;
                 }
-                S.stack[2 * depth][lane] = cur;             // entry bits
-                S.fend[depth] = end;
-                S.felse[depth] = sk == AMC_T_IF ? e : -1;
-                ++depth;
-                cur = 0;                                     // the branch / body from scratch
-                ++pos;
-            } else if (sk == AMC_T_ELSE) {
-                if (!depth || S.felse[depth - 1] != pos) {
-                    malformed = true;
-                    break;
-                }
-                S.stack[2 * (depth - 1) + 1][lane] = cur;   // then-branch bits
-                cur = 0;
-                ++pos;
-            } else if (sk == AMC_T_END) {
-                if (!depth || S.fend[depth - 1] != pos) {
-                    malformed = true;
-                    break;
-                }
-                --depth;
-                const uint64_t entry = S.stack[2 * depth][lane];
-                cur = S.felse[depth] >= 0 ? (entry | (S.stack[2 * depth + 1][lane] & cur)) : entry;
-                ++pos;
-            } else {
-                malformed = true;                            // pw / GT / EN, or a byte out of range
-                break;
+                __syncwarp();
             }
-            __syncwarp();
         }
-        if (depth) malformed = true;
+        malformed = depth || stop != NONE;
         if (malformed) break;
         // W obligations whose tracked bits fall in this window
         for (int j = 0; j < nd; ++j) {
             const int64_t b0 = S.base[j];
             if (b0 < 0) continue;
-            const int32_t aj = S.arr[j];
-            const int64_t n = p.arr_loc_off[aj + 1] - p.arr_loc_off[aj];
-            const int64_t lo = max(b0, w0) - w0, hi = min(b0 + n, w0 + window) - w0;
+            const int64_t lo = max(b0, w0) - w0, hi = min(b0 + S.locs[j], w0 + window) - w0;
             if (lo >= hi) continue;
-            // bits [lo, hi) of the window: lane words [64 lane, 64 lane + 64)
-            const int64_t wlo = (int64_t)lane * 64, whi = wlo + 64;
-            const int64_t a0 = max(lo, wlo), a1 = min(hi, whi);
-            bool miss = false;
-            if (a0 < a1) {
-                const int s0 = (int)(a0 - wlo), s1 = (int)(a1 - wlo);
-                const uint64_t need = (s1 - s0 == 64) ? ~0ull : (((1ull << (s1 - s0)) - 1ull) << s0);
-                miss = (cur & need) != need;
+            bool miss = false;                                         // bits [lo, hi) of the window
+            for (int64_t i = lo / 32 + lane; i * 32 < hi; i += 32) {
+                uint32_t need = ~0u;
+                if (i * 32 < lo) need &= ~0u << (lo - i * 32);
+                if (i * 32 + 32 > hi) need &= ~0u >> (i * 32 + 32 - hi);
+                miss |= (S.cur[i] & need) != need;
             }
             if (__any_sync(0xffffffffu, miss)) {
                 viol |= 8u;
-                unmet = min(unmet, aj);
+                unmet = min(unmet, S.arr[j]);
             }
         }
+        __syncwarp();
     }
+    if (range < stop) raise_error(p.err, AMC_E_RANGE);
+    __syncwarp();
     if (malformed) {
         if (lane == 0) raise_error(p.err, AMC_E_INVALID);
         return;
     }
     // combine the lanes' findings
     viol = __reduce_or_sync(0xffffffffu, viol);
+    if (__any_sync(0xffffffffu, bad != NONE))
 #pragma unroll
-    for (int d = 16; d; d >>= 1) bad = min(bad, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)bad, d));
+        for (int d = 16; d; d >>= 1) bad = min(bad, __shfl_xor_sync(0xffffffffu, bad, d));
     unmet = __reduce_min_sync(0xffffffffu, unmet);
     if (lane == 0) {
         p.violations[c] = viol;
-        p.first_bad[c] = bad == INT64_MAX ? -1 : bad;
+        p.first_bad[c] = bad == NONE ? -1 : (int64_t)bad;
         p.first_unmet[c] = unmet == INT32_MAX ? -1 : unmet;
     }
 }
@@ -259,13 +304,28 @@ __global__ void __launch_bounds__(WD_WARPS * 32) wd_kernel(const WdParams p)
     __shared__ WdWarp S[WD_WARPS];
     const int w = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
+    // WD_CLAIM calls per claim: their extents in one load
+    const int64_t n_locs = p.n_arrays > 0 ? p.arr_loc_off[p.n_arrays] : 0;
     for (;;) {
-        long long c = 0;
-        if (lane == 0) c = (long long)atomicAdd(p.queue, 1ull);
-        c = __shfl_sync(0xffffffffu, c, 0);
-        if (c >= p.n_calls) break;
-        wd_call(p, c, S[w]);
-        __syncwarp();
+        long long c0 = 0;
+        if (lane == 0) c0 = (long long)atomicAdd(p.queue, (unsigned long long)WD_CLAIM);
+        c0 = __shfl_sync(0xffffffffu, c0, 0);
+        if (c0 >= p.n_calls) break;
+        const int n = (int)min((int64_t)WD_CLAIM, p.n_calls - (int64_t)c0);
+        const long long to = lane <= n ? p.call_tok_off[c0 + lane] : 0, mo = lane <= n ? p.call_am_off[c0 + lane] : 0;
+        for (int i = 0; i < n; ++i) {
+            const int64_t t0 = __shfl_sync(0xffffffffu, to, i), t1 = __shfl_sync(0xffffffffu, to, i + 1);
+            const int64_t m0 = __shfl_sync(0xffffffffu, mo, i), m1 = __shfl_sync(0xffffffffu, mo, i + 1);
+            if (t0 < 0 || t1 < t0 || t1 > p.n_tokens || m0 < 0 || m1 < m0 || m1 > p.n_decls ||
+                m1 - m0 > AMC_WD_MAX_DECLS) {
+                if (lane == 0) raise_error(p.err, AMC_E_INVALID);
+            } else if (t1 - t0 < INT32_MAX - 64) {
+                wd_call<int32_t>(p, c0 + i, t0, (int32_t)(t1 - t0), m0, (int)(m1 - m0), n_locs, S[w]);
+            } else {
+                wd_call<int64_t>(p, c0 + i, t0, t1 - t0, m0, (int)(m1 - m0), n_locs, S[w]);
+            }
+            __syncwarp();
+        }
     }
 }
 
@@ -298,8 +358,8 @@ int launch_well_declared(const WdLaunch& L, cudaStream_t s)
     int dev = 0, n_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t need = (L.n_calls + WD_WARPS - 1) / WD_WARPS;
-    const int grid = (int)(need < (int64_t)n_sm * 8 ? need : (int64_t)n_sm * 8);
+    const int64_t need = (L.n_calls + WD_WARPS * WD_CLAIM - 1) / (WD_WARPS * WD_CLAIM);
+    const int grid = (int)(need < (int64_t)n_sm * 10 ? need : (int64_t)n_sm * 10);
     if (L.profile & 1) profile_begin(s);
     wd_kernel<<<grid, WD_WARPS * 32, 0, s>>>(p);
     if (L.profile & 2) profile_end(s);
