@@ -876,13 +876,14 @@ def measure_programs(args, amc, dev):
 
 
 def batch_launches(n_tokens):
-    """Kernels of one batched relation-mode check (longest-first queue):
-    bucket count, scan and order; when the batch is longer than the split
-    length (so that some program may be split) also the slot offsets, the
-    cuts, the relation reset, the ordered unit offsets, the reduce phase and
-    the carry; then the apply phase."""
+    """Kernels of one batched relation-mode check (costliest-first queue):
+    bucket count, scan and order, the programs evaluated variable by variable,
+    and the token-by-token kernels for the rest, which end at once when there
+    is none: the apply phase, and when the batch is longer than the split
+    length the slot offsets, the cuts, the relation reset, the ordered unit
+    offsets, the reduce phase and the carry."""
     split = int(os.environ.get("AMC_BATCH_SPLIT", "65536"))
-    return 3 + 1 if n_tokens <= split else 3 + 3 + 1 + 1 + 1 + 1
+    return 3 + 1 + 1 if n_tokens <= split else 3 + 1 + 3 + 1 + 1 + 1 + 1
 
 
 def measure_guarded(args, amc, dev):

@@ -8,6 +8,11 @@
 // A program's "first fault" is the smallest token of an op whose possible
 // pre-statuses include a non-stuck status that the op makes stuck.
 //
+// Programs of at most 65,535 tokens over at most 4,096 variables (and no longer
+// than the split length) are evaluated variable by variable (batch_vars.cu).
+// The rest -- long programs, and launches without construct rows -- is done
+// here, token by token for all variables at once.
+//
 // Work is split by op count.  A program longer than the split length (with at
 // most SPLIT_VARS variables) is cut into segments of about that length at
 // top-level boundaries (never inside an If or While); every other program is
@@ -310,7 +315,10 @@ struct Plan {
     uint8_t* rsave;               // [reduce warps][2][AMC_MAX_DEPTH][seg_max] reduce-pass copies
     int64_t* ord_off;             // [P + 1] apply units before the k-th program of the queue order
     int simple;                   // no program can be split: one unit per program, no planning
+    const int* gate;              // nullable: set when a program is left to these kernels (else they do nothing)
 };
+
+__device__ __forceinline__ bool gated_off(const int* gate) { return gate && *gate == 0; }
 
 __device__ __forceinline__ int64_t split_slots(int64_t len, int32_t nv, int64_t split)
 {
@@ -354,6 +362,7 @@ __global__ void __launch_bounds__(BWARPS * 32, MINB) batch_kernel(const BatchPar
 {
     __shared__ WarpSmem smem[BWARPS];
     __shared__ TabSmem tab;
+    if (gated_off(pl.gate)) return;
     const int w = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     WarpSmem& S = smem[w];
@@ -430,6 +439,7 @@ __global__ void __launch_bounds__(BWARPS * 32, MINB) batch_kernel(const BatchPar
             if (lane == 0) raise_error(p.err, AMC_E_INVALID);
             continue;
         }
+        if (pl.gate && program_fits_vars(pt1 - pt0, nv, p.split)) continue;     // evaluated variable by variable
         if (nv <= SMEM_VARS)
             run_unit<true>(p, u, S, tab);
         else
@@ -444,8 +454,10 @@ __global__ void __launch_bounds__(1024) plan_offsets_kernel(const int64_t* __res
                                                             const int32_t* __restrict__ nvars, int64_t P,
                                                             int64_t* __restrict__ slot_off,
                                                             int64_t* __restrict__ unit_off,
-                                                            int64_t* __restrict__ prog_ff, int64_t split)
+                                                            int64_t* __restrict__ prog_ff, int64_t split,
+                                                            const int* gate)
 {
+    if (gated_off(gate)) return;
     __shared__ unsigned long long tmp_s[32], tmp_u[32];
     __shared__ unsigned long long carry_s, carry_u;
     if (threadIdx.x == 0) {
@@ -506,8 +518,9 @@ __global__ void __launch_bounds__(1024) plan_offsets_kernel(const int64_t* __res
 // warp prefix sum of +1 (IF, WHILE) / -1 (END) over 32 tokens at a time.
 __global__ void plan_cuts_kernel(const uint8_t* __restrict__ tok, const int64_t* __restrict__ tok_off,
                                  const int32_t* __restrict__ nvars, int64_t P, const int64_t* __restrict__ slot_off,
-                                 int64_t* __restrict__ seg_t0, int64_t split)
+                                 int64_t* __restrict__ seg_t0, int64_t split, const int* gate)
 {
+    if (gated_off(gate)) return;
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t pr = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; pr < P; pr += nw) {
@@ -567,18 +580,36 @@ __global__ void plan_cuts_kernel(const uint8_t* __restrict__ tok, const int64_t*
     }
 }
 
-// Queue order of the apply phase: programs by decreasing length bucket
-// (floor(log2(tokens))); the order within a bucket is whatever the cursors
-// give (it only decides which warp starts which program first).
-__device__ __forceinline__ int len_bucket(int64_t len) { return len <= 0 ? 63 : 63 - (64 - __clzll(len)); }
+// Queue order: programs by decreasing cost, four buckets per power of two from
+// 2^8 on; the order within a bucket is whatever the cursors give (it only
+// decides which warp starts which program first).  A program costs its length
+// and more the fewer its variables are (ops that share a construct with another
+// op of their variable run again with it, and few chains keep few lanes busy):
+// by length alone the last programs kept a 100,000-program batch 2.5 ms longer.
+__device__ __forceinline__ int cost_bucket(int64_t len, int32_t nv)
+{
+    if (len <= 0) return 63;
+    const uint64_t x = (uint64_t)len * (uint64_t)(4 + min(4800 / max(nv, 1), 64)) / 4;
+    const int e = 63 - __clzll((long long)x);
+    const int k = 4 * e + (e >= 2 ? (int)(x >> (e - 2)) & 3 : 0) - 32;
+    return 62 - min(max(k, 0), 62);
+}
 
-__global__ void bucket_count_kernel(const int64_t* __restrict__ tok_off, int64_t n, int32_t* __restrict__ counts)
+// With `others`, also notes whether a program is not evaluated variable by
+// variable.
+__global__ void bucket_count_kernel(const int64_t* __restrict__ tok_off, const int32_t* __restrict__ nvars, int64_t n,
+                                    int32_t* __restrict__ counts, int64_t split, int* others)
 {
     __shared__ int32_t c[64];
     if (threadIdx.x < 64) c[threadIdx.x] = 0;
     __syncthreads();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&c[len_bucket(tok_off[i + 1] - tok_off[i])], 1);
+    bool other = false;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t len = tok_off[i + 1] - tok_off[i];
+        atomicAdd(&c[cost_bucket(len, nvars[i])], 1);
+        other |= !program_fits_vars(len, nvars[i], split);
+    }
+    if (others && other) *others = 1;
     __syncthreads();
     if (threadIdx.x < 64 && c[threadIdx.x]) atomicAdd(&counts[threadIdx.x], c[threadIdx.x]);
 }
@@ -596,12 +627,13 @@ __global__ void bucket_scan_kernel(int32_t* __restrict__ counts, int64_t* __rest
     }
 }
 
-__global__ void order_kernel(const int64_t* __restrict__ tok_off, int64_t n, const int64_t* __restrict__ boff,
+__global__ void order_kernel(const int64_t* __restrict__ tok_off, const int32_t* __restrict__ nvars, int64_t n,
+                             const int64_t* __restrict__ boff,
                              int32_t* __restrict__ cursor, int32_t* __restrict__ order)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const int b = len_bucket(tok_off[i + 1] - tok_off[i]);
+    const int b = cost_bucket(tok_off[i + 1] - tok_off[i], nvars[i]);
     order[boff[b] + atomicAdd(&cursor[b], 1)] = (int32_t)i;
 }
 
@@ -609,8 +641,9 @@ __global__ void order_kernel(const int64_t* __restrict__ tok_off, int64_t n, con
 // the queue order (exclusive scan).
 __global__ void __launch_bounds__(1024) order_units_kernel(const int32_t* __restrict__ order,
                                                            const int64_t* __restrict__ unit_off, int64_t P,
-                                                           int64_t* __restrict__ ord_off)
+                                                           int64_t* __restrict__ ord_off, const int* gate)
 {
+    if (gated_off(gate)) return;
     __shared__ unsigned long long tmp[32];
     __shared__ unsigned long long carry;
     if (threadIdx.x == 0) carry = 0;
@@ -645,6 +678,7 @@ __global__ void __launch_bounds__(1024) order_units_kernel(const int32_t* __rest
 // relations of the ones before (image of the set through the 25-bit rows).
 __global__ void carry_kernel(const BatchParams p, const Plan pl)
 {
+    if (gated_off(pl.gate)) return;
     // program by block, variable by thread
     for (int64_t pr = blockIdx.x; pr < p.n_progs; pr += gridDim.x) {
         const int64_t s0 = pl.slot_off[pr], s1 = pl.slot_off[pr + 1];
@@ -668,6 +702,7 @@ __global__ void carry_kernel(const BatchParams p, const Plan pl)
 
 __global__ void zero_rel_kernel(const BatchParams p, const Plan pl)
 {
+    if (gated_off(pl.gate)) return;
     const int64_t n = pl.slot_off[p.n_progs] * (int64_t)SPLIT_VARS;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) pl.R[i] = 0;
@@ -771,31 +806,45 @@ int launch_batch(const BatchLaunch& B, cudaStream_t s)
         const int64_t need = (B.n_progs + BWARPS - 1) / BWARPS;
         if (grid > need) grid = need;
     }
+    // the programs that fit are evaluated variable by variable (its rows of 8
+    // bytes a token are the save and alt rows); the kernels below take the rest,
+    // and nothing when there is none
+    const bool by_vars = p.save_rows == AMC_MAX_DEPTH;
+    unsigned long long* vars_queue = reinterpret_cast<unsigned long long*>(p.queue_head) + 1;
+    int* others = reinterpret_cast<int*>(p.queue_head + 2);
+    pl.gate = by_vars ? others : nullptr;
     if (B.profile & 1) profile_begin(s);
+    if (cudaMemsetAsync(p.queue_head, 0, 24, s) != cudaSuccess) return AMC_E_CUDA;
+    if (cudaMemsetAsync(counts, 0, 256, s) != cudaSuccess) return AMC_E_CUDA;
+    if (B.longest_first || by_vars)
+        bucket_count_kernel<<<128, 256, 0, s>>>(B.prog_tok_off, B.prog_nvars, B.n_progs, counts, p.split,
+                                                by_vars ? others : nullptr);
     if (!pl.simple) {
         plan_offsets_kernel<<<1, 1024, 0, s>>>(B.prog_tok_off, B.prog_nvars, B.n_progs,
                                                const_cast<int64_t*>(pl.slot_off), const_cast<int64_t*>(pl.unit_off),
-                                               B.prog_first_fault, p.split);
+                                               B.prog_first_fault, p.split, pl.gate);
         plan_cuts_kernel<<<n_sm * 4, 256, 0, s>>>(B.tok, B.prog_tok_off, B.prog_nvars, B.n_progs, pl.slot_off,
-                                                  pl.seg_t0, p.split);
+                                                  pl.seg_t0, p.split, pl.gate);
         zero_rel_kernel<<<n_sm * 4, 256, 0, s>>>(p, pl);
     }
     if (B.longest_first) {
-        if (cudaMemsetAsync(counts, 0, 256, s) != cudaSuccess) return AMC_E_CUDA;
-        bucket_count_kernel<<<128, 256, 0, s>>>(B.prog_tok_off, B.n_progs, counts);
         bucket_scan_kernel<<<1, 32, 0, s>>>(counts, boff);
-        order_kernel<<<(unsigned)((B.n_progs + 255) / 256), 256, 0, s>>>(B.prog_tok_off, B.n_progs, boff, counts,
-                                                                           order);
-        if (!pl.simple) order_units_kernel<<<1, 1024, 0, s>>>(order, pl.unit_off, B.n_progs, pl.ord_off);
+        order_kernel<<<(unsigned)((B.n_progs + 255) / 256), 256, 0, s>>>(B.prog_tok_off, B.prog_nvars, B.n_progs, boff,
+                                                                           counts, order);
+        if (!pl.simple)
+            order_units_kernel<<<1, 1024, 0, s>>>(order, pl.unit_off, B.n_progs, pl.ord_off, pl.gate);
         p.order = order;
     }
+    if (by_vars) {
+        const int rc = launch_batch_vars(p, B.max_ctas, vars_queue, s);
+        if (rc) return rc;
+    }
     if (!pl.simple) {
-        if (cudaMemsetAsync(p.queue_head, 0, 8, s) != cudaSuccess) return AMC_E_CUDA;
         const int64_t rgrid = grid < L.red_ctas ? grid : L.red_ctas;
         if (rgrid > 0) kern<<<(unsigned)rgrid, BWARPS * 32, 0, s>>>(p, pl, 0);      // reduce
         carry_kernel<<<n_sm * 4, 256, 0, s>>>(p, pl);
+        if (cudaMemsetAsync(p.queue_head, 0, 8, s) != cudaSuccess) return AMC_E_CUDA;
     }
-    if (cudaMemsetAsync(p.queue_head, 0, 8, s) != cudaSuccess) return AMC_E_CUDA;
     kern<<<(unsigned)grid, BWARPS * 32, 0, s>>>(p, pl, 1);       // apply
     if (B.profile & 2) profile_end(s);
     return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;

@@ -49,6 +49,31 @@ struct BatchLaunch {
     int profile = 0;
 };
 
+// Programs evaluated variable by variable (batch_vars.cu): positions fit 16
+// bits and the variables' last ops a warp's share of shared memory.
+constexpr int32_t VARS_MAX_NV = 4096;
+constexpr int64_t VARS_MAX_LEN = 65535;
+__device__ __forceinline__ bool program_fits_vars(int64_t len, int32_t nv, int64_t split)
+{
+    return len <= VARS_MAX_LEN && len <= split && nv <= VARS_MAX_NV;
+}
+// Whether that is done for program `prog`: reported and left out when its
+// extents are malformed.
+__device__ __forceinline__ bool program_by_vars(const BatchParams& p, int64_t prog)
+{
+    const int64_t a = p.prog_tok_off[prog], b = p.prog_tok_off[prog + 1];
+    const int32_t nv = p.prog_nvars[prog];
+    if (a < 0 || b < a || b > p.n_tokens || nv < 0 || p.prog_var_off[prog] < 0 ||
+        p.prog_var_off[prog + 1] - p.prog_var_off[prog] != nv) {
+        if ((threadIdx.x & 31) == 0) raise_error(p.err, AMC_E_INVALID);
+        return false;
+    }
+    return program_fits_vars(b - a, nv, p.split);
+}
+// Those programs of the batch (p.save / p.alt with AMC_MAX_DEPTH rows: 8 bytes
+// a token each); *queue is zero.
+int launch_batch_vars(const BatchParams& p, int64_t max_ctas, unsigned long long* queue, cudaStream_t s);
+
 size_t batch_workspace_bytes(int64_t n_tokens, int64_t n_progs);
 size_t batch_workspace_bytes(int64_t n_tokens, int64_t n_progs, bool no_split, int save_rows);
 int launch_batch(const BatchLaunch& B, cudaStream_t s);
