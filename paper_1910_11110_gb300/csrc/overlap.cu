@@ -78,7 +78,7 @@ __global__ void ov_sweep_kernel(const OvParams p)
     const int64_t pos = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (pos >= p.A) return;
-    if (FILL && p.off[p.A] > p.cap) return;                  // over capacity: reported by the count pass
+    if (FILL && p.off[(int64_t)p.A * p.nb] > p.cap) return;  // over capacity: reported by the count pass
     const int32_t i = (int32_t)p.sval[pos];
     const int64_t e = (int64_t)p.start[i] + p.len[i];
     const int32_t ub = upper_pos(p.skey, (int32_t)pos, p.A, e);
@@ -88,7 +88,9 @@ __global__ void ov_sweep_kernel(const OvParams p)
         // the shared part of the two lifetimes, and its buckets
         const int32_t lo = p.born ? max(bi, p.born[j]) : 0, hi = p.born ? min(di, p.died[j]) : 1;
         if (lo >= hi) continue;
-        const int32_t b0 = p.born ? (int32_t)(lo / p.bl) : 0, b1 = p.born ? (int32_t)((hi - 1) / p.bl) : 0;
+        // (a malformed lifetime, reported elsewhere, stays within its array's lists)
+        const int32_t b0 = p.born ? (int32_t)(max(lo, 0) / p.bl) : 0;
+        const int32_t b1 = p.born ? (int32_t)min((hi - 1) / p.bl, (int64_t)p.nb - 1) : 0;
         for (int32_t b = b0; b <= b1; ++b) {
             const int64_t li = (int64_t)i * p.nb + b, lj = (int64_t)j * p.nb + b;
             if (FILL) {
