@@ -7,8 +7,20 @@
 // the overlapping arrays whose lifetime meets a's within bucket b, so that a
 // call at c reads list (a, c / bucket_len) -- about the arrays live near c,
 // not every array that ever overlaps a -- and keeps the entries live at c:
-// r_v as the paper queries it at that call.  Sort and sweep, O(A log A + P)
-// for P listed entries:
+// r_v as the paper queries it at that call.
+//
+// Without lifetimes and up to OV_DIRECT arrays the lists are counted and filled
+// by testing all pairs: a warp per array takes the other arrays 32 at a time in
+// ascending order and a ballot places the matches, so that the lists come out
+// ascending and nothing is sorted: seven kernels instead of 37.  All pairs is
+// A^2 / 32 warp steps of about ten instructions, which a sort overtakes: a whole
+// translation of 20,000 calls over 1,024 / 4,096 / 8,192 / 12,288 arrays took
+// 145 / 198 / 339 / 1080 us so and 297 / 322 / 355 / 716 us by the sort.  (With
+// lifetimes all pairs lose: an array that lives long meets thousands of others,
+// each in many buckets, and its one warp or CTA appends them one after another;
+// counting 16,384 arrays over 16 vectors took 1.6 ms so, 0.2 by the sort.)
+//
+// Otherwise, sort and sweep, O(A log A + P) for P listed entries:
 //   1. the arrays sorted by range start (stable LSD radix sort, ids as values);
 //   2. a warp per sorted position p: the arrays after p whose start lies below
 //      p's end overlap it (they start no earlier and have at least one
@@ -72,6 +84,13 @@ __device__ __forceinline__ int32_t upper_pos(const uint32_t* skey, int32_t lo, i
     return a;
 }
 
+// The arrays after a position are dealt to OV_SPLIT warps, 32 at a time in turn,
+// and a warp has the cursors of OV_STEP buckets on their way at once: one warp
+// alone, a bucket after another, waited out the atomics of an array that meets a
+// thousand others (16 vectors, 16,384 pvectors: 66 us counting, 958 us
+// filling; 30 and 107 us so).
+constexpr int OV_SPLIT = 8;
+constexpr int OV_STEP = 4;
 template <bool FILL>
 __global__ void ov_sweep_kernel(const OvParams p)
 {
@@ -81,9 +100,11 @@ __global__ void ov_sweep_kernel(const OvParams p)
     if (FILL && p.off[(int64_t)p.A * p.nb] > p.cap) return;  // over capacity: reported by the count pass
     const int32_t i = (int32_t)p.sval[pos];
     const int64_t e = (int64_t)p.start[i] + p.len[i];
-    const int32_t ub = upper_pos(p.skey, (int32_t)pos, p.A, e);
+    const int64_t first = pos + 1 + (int64_t)blockIdx.y * 32;
+    if (first >= p.A || (int64_t)p.skey[first] >= e) return;
+    const int32_t ub = upper_pos(p.skey, (int32_t)first, p.A, e);
     const int32_t bi = p.born ? p.born[i] : 0, di = p.born ? p.died[i] : 1;
-    for (int32_t q = (int32_t)pos + 1 + lane; q < ub; q += 32) {
+    for (int64_t q = first + lane; q < ub; q += 32 * OV_SPLIT) {
         const int32_t j = (int32_t)p.sval[q];
         // the shared part of the two lifetimes, and its buckets
         const int32_t lo = p.born ? max(bi, p.born[j]) : 0, hi = p.born ? min(di, p.died[j]) : 1;
@@ -91,19 +112,25 @@ __global__ void ov_sweep_kernel(const OvParams p)
         // (a malformed lifetime, reported elsewhere, stays within its array's lists)
         const int32_t b0 = p.born ? (int32_t)(max(lo, 0) / p.bl) : 0;
         const int32_t b1 = p.born ? (int32_t)min((hi - 1) / p.bl, (int64_t)p.nb - 1) : 0;
-        for (int32_t b = b0; b <= b1; ++b) {
-            const int64_t li = (int64_t)i * p.nb + b, lj = (int64_t)j * p.nb + b;
-            if (FILL) {
-                const int64_t wi = p.off[li] + atomicAdd(&p.cnt[li], 1);
-                const int64_t wj = p.off[lj] + atomicAdd(&p.cnt[lj], 1);
-                p.pkey[wi] = (uint32_t)j;
-                p.pval[wi] = (uint32_t)li;
-                p.pkey[wj] = (uint32_t)i;
-                p.pval[wj] = (uint32_t)lj;
-            } else {
-                atomicAdd(&p.cnt[li], 1);
-                atomicAdd(&p.cnt[lj], 1);
-            }
+        for (int32_t b = b0; b <= b1; b += OV_STEP) {
+            int32_t ni[OV_STEP], nj[OV_STEP];
+#pragma unroll
+            for (int k = 0; k < OV_STEP; ++k)
+                if (b + k <= b1) {
+                    ni[k] = atomicAdd(&p.cnt[(int64_t)i * p.nb + b + k], 1);
+                    nj[k] = atomicAdd(&p.cnt[(int64_t)j * p.nb + b + k], 1);
+                }
+            if (!FILL) continue;
+#pragma unroll
+            for (int k = 0; k < OV_STEP; ++k)
+                if (b + k <= b1) {
+                    const int64_t li = (int64_t)i * p.nb + b + k, lj = (int64_t)j * p.nb + b + k;
+                    const int64_t wi = p.off[li] + ni[k], wj = p.off[lj] + nj[k];
+                    p.pkey[wi] = (uint32_t)j;
+                    p.pval[wi] = (uint32_t)li;
+                    p.pkey[wj] = (uint32_t)i;
+                    p.pval[wj] = (uint32_t)lj;
+                }
         }
     }
 }
@@ -147,6 +174,37 @@ __global__ void ov_copy_kernel(const uint32_t* __restrict__ other, const uint32_
         dst[i] = y << 1 | (uint32_t)(sx <= sy && (int64_t)sy + p.len[y] <= (int64_t)sx + p.len[x]);
     }
 }
+
+// All pairs: list lengths (FILL = false) or the lists themselves.
+template <bool FILL>
+__global__ void __launch_bounds__(256) ov_direct_kernel(const OvParams p, uint32_t* __restrict__ idx)
+{
+    const int lane = threadIdx.x & 31;
+    const int32_t a = (int32_t)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (a >= p.A) return;
+    if (FILL && p.off[p.A] > p.cap) return;                // over capacity: reported by the count pass
+    const int32_t s = p.start[a], l = p.len[a];
+    if (!FILL && lane == 0 && (s < 0 || l < 1 || (int64_t)s + l > INT32_MAX)) raise_error(p.err, AMC_E_INVALID);
+    const int64_t e = (int64_t)s + l;
+    int64_t at = FILL ? p.off[a] : 0;
+    for (int32_t j0 = 0; j0 < p.A; j0 += 32) {
+        const int32_t j = j0 + lane;
+        bool hit = false, inside = false;
+        if (j < p.A && j != a) {
+            const int32_t sj = p.start[j];
+            const int64_t ej = (int64_t)sj + p.len[j];
+            hit = sj < e && s < ej;
+            inside = s <= sj && ej <= e;
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, hit);
+        if (FILL && hit) idx[at + __popc(m & lanemask_lt())] = (uint32_t)j << 1 | inside;
+        at += __popc(m);
+    }
+    if (!FILL && lane == 0) p.cnt[a] = (int32_t)at;
+}
+
+// Most arrays whose pairs are all tested.
+constexpr int32_t OV_DIRECT = 8192;
 
 struct OvLayout {
     size_t k0, v0, k1, v1, sscr, cnt, scan, gate, p0, p1, p2, p3, pscr, total;
@@ -223,6 +281,19 @@ int launch_overlaps(const OverlapBuild& O, cudaStream_t s)
     p.err = O.err;
     const unsigned ab = (unsigned)((A + 255) / 256);
     const unsigned lb = (unsigned)((NL + 256) / 256);
+    if (!O.arr_born && A <= OV_DIRECT) {
+        int* gate = reinterpret_cast<int*>(w + L.gate);
+        const unsigned wb = (unsigned)((A + 7) / 8);
+        ov_direct_kernel<false><<<wb, 256, 0, s>>>(p, nullptr);
+        int rc = dscan_exclusive(p.cnt, O.ov_off, NL, w + L.scan, s);
+        if (rc) return rc;
+        ov_total_kernel<<<1, 1, 0, s>>>(O.ov_off, NL, O.cap, O.n_pairs, O.err, gate);
+        if (O.cap > 0 && O.ov_idx) {
+            ov_direct_kernel<true><<<wb, 256, 0, s>>>(p, O.ov_idx);
+            ov_clear_kernel<<<lb, 256, 0, s>>>(O.ov_off, NL, gate);
+        }
+        return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
+    }
     ov_keys_kernel<<<ab, 256, 0, s>>>(O.arr_start, O.arr_len, A, k[0], v[0], O.err);
     ov_zero_kernel<<<lb, 256, 0, s>>>(p.cnt, NL);
     int passes = 0;
@@ -232,7 +303,7 @@ int launch_overlaps(const OverlapBuild& O, cudaStream_t s)
     p.skey = k[passes & 1];
     p.sval = v[passes & 1];
     const unsigned wb = (unsigned)(((int64_t)A * 32 + 255) / 256);
-    ov_sweep_kernel<false><<<wb, 256, 0, s>>>(p);
+    ov_sweep_kernel<false><<<dim3(wb, OV_SPLIT), 256, 0, s>>>(p);
     rc = dscan_exclusive(p.cnt, O.ov_off, NL, w + L.scan, s);
     if (rc) return rc;
     int* gate = reinterpret_cast<int*>(w + L.gate);
@@ -243,7 +314,7 @@ int launch_overlaps(const OverlapBuild& O, cudaStream_t s)
     uint32_t* pv[2] = {reinterpret_cast<uint32_t*>(w + L.p2), reinterpret_cast<uint32_t*>(w + L.p3)};
     p.pkey = pk[0];
     p.pval = pv[0];
-    ov_sweep_kernel<true><<<wb, 256, 0, s>>>(p);
+    ov_sweep_kernel<true><<<dim3(wb, OV_SPLIT), 256, 0, s>>>(p);
     // by other, then (stably) by owner list; the count is read on the device
     const int64_t* n_dev = O.ov_off + NL;
     rc = launch_ss_radix(pk, pv, n_dev, O.cap, A, w + L.pscr, gate, s, &passes);
