@@ -23,6 +23,7 @@ struct PsParams {
     uint32_t* save;                // [AMC_MAX_DEPTH][2][total_vars] construct copies
     const int32_t* order;
     uint64_t* queue_head;
+    const int64_t* n_long;         // programs at the front of the order that several warps share
     int* err;
     SetTables tab;
 };
