@@ -44,6 +44,7 @@ __device__ long long block_excl_sum64(long long x, long long* tmp, long long* to
 __global__ void __launch_bounds__(SCAN_NT) scan_reduce(const int32_t* __restrict__ in, int64_t n,
                                                        long long* __restrict__ block_sums)
 {
+    follow();
     __shared__ long long tmp[SCAN_NT / 32 + 1];
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
     long long s = 0;
@@ -58,6 +59,7 @@ __global__ void __launch_bounds__(SCAN_NT) scan_reduce(const int32_t* __restrict
 
 __global__ void __launch_bounds__(SCAN_NT) scan_top(long long* __restrict__ block_sums, int64_t n_blocks)
 {
+    follow();
     __shared__ long long tmp[SCAN_NT / 32 + 1];
     long long carry = 0;
     for (int64_t lo = 0; lo < n_blocks; lo += SCAN_NT) {
@@ -75,6 +77,7 @@ __global__ void __launch_bounds__(SCAN_NT) scan_apply(const int32_t* __restrict_
                                                       const long long* __restrict__ block_sums,
                                                       int64_t* __restrict__ out, int64_t n_blocks)
 {
+    follow();
     __shared__ long long tmp[SCAN_NT / 32 + 1];
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_IPT;
     long long v[SCAN_IPT];
@@ -112,9 +115,9 @@ int dscan_exclusive(const int32_t* in, int64_t* out, int64_t n, void* workspace,
         if (cudaMemsetAsync(out, 0, 8, s) != cudaSuccess) return AMC_E_CUDA;
         return AMC_OK;
     }
-    scan_reduce<<<(unsigned)nb, SCAN_NT, 0, s>>>(in, n, bs);
-    scan_top<<<1, SCAN_NT, 0, s>>>(bs, nb);
-    scan_apply<<<(unsigned)nb, SCAN_NT, 0, s>>>(in, n, bs, out, nb);
+    chain(scan_reduce, (unsigned)nb, SCAN_NT, 0, s)(in, n, bs);
+    chain(scan_top, 1, SCAN_NT, 0, s)(bs, nb);
+    chain(scan_apply, (unsigned)nb, SCAN_NT, 0, s)(in, n, bs, out, nb);
     return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
 }
 

@@ -109,6 +109,7 @@ __global__ void kl_keys_kernel(const uint8_t* __restrict__ op, const int32_t* __
                                uint8_t* __restrict__ step, const uint8_t* __restrict__ init, uint8_t* __restrict__ fin,
                                int32_t* __restrict__ vff, int64_t* ff, int* err)
 {
+    follow();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (int64_t i = g; i < n; i += stride) {
@@ -139,6 +140,7 @@ __global__ void kl_keys_kernel(const uint8_t* __restrict__ op, const int32_t* __
 // bit v: variable v is stuck
 __global__ void kl_bitmap_kernel(const uint8_t* __restrict__ st, int32_t n_vars, uint32_t* __restrict__ bm)
 {
+    follow();
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t m = __ballot_sync(0xffffffffu, v < n_vars && st[v] == KL_F);
     if ((threadIdx.x & 31) == 0 && v < n_vars) bm[v >> 5] = m;
@@ -164,6 +166,7 @@ struct KFilterParams {
 // threads an SM stream beside the 128 KB bitmap.
 __global__ void __launch_bounds__(KFT, 1) kl_filter_kernel(const __grid_constant__ KFilterParams p)
 {
+    follow();
     extern __shared__ __align__(16) uint32_t sbm[];
     __shared__ uint32_t valid[8];
     const int t = threadIdx.x, lane = t & 31;
@@ -241,6 +244,7 @@ __global__ void __launch_bounds__(256) kl_compact_kernel(const uint32_t* __restr
                                                          int64_t ns, uint32_t* __restrict__ key,
                                                          uint32_t* __restrict__ val)
 {
+    follow();
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < ns; s += nw) {
@@ -274,6 +278,7 @@ struct KSegParams {
 
 __global__ void __launch_bounds__(KNT) kl_seg_kernel(const KSegParams p)
 {
+    follow();
     __shared__ uint32_t wtot[KNT / 32];
     __shared__ uint32_t s_tile, s_carry;
     const int64_t n = p.n_dev ? max((int64_t)0, min(*p.n_dev, p.cap)) : p.cap;
@@ -454,7 +459,7 @@ int launch_kloc(const KlocLaunch& L, cudaStream_t s)
     const int64_t blocks = (work + 255) / 256;
     const int kgrid = (int)(blocks < (int64_t)n_sm * 8 ? (blocks > 0 ? blocks : 1) : (int64_t)n_sm * 8);
     const int pack = L.n_vars <= (1 << KOP_SHIFT) ? 1 : 0;
-    kl_keys_kernel<<<kgrid, 256, 0, s>>>(L.op, L.var, first, L.n_vars, L.k, pack, key[0], val[0], L.step, L.init,
+    chain(kl_keys_kernel, kgrid, 256, 0, s)(L.op, L.var, first, L.n_vars, L.k, pack, key[0], val[0], L.step, L.init,
                                          L.final_status, L.vff, L.first_fault, L.err);
     if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
     // the pairs in key[0] / val[0] (n of them, or *n_dev of at most n), from the
@@ -483,7 +488,7 @@ int launch_kloc(const KlocLaunch& L, cudaStream_t s)
         p.err = L.err;
         p.bm = n_dev ? bm : nullptr;
         const int sgrid = (int)(tiles < (int64_t)n_sm * 8 ? tiles : (int64_t)n_sm * 8);
-        kl_seg_kernel<<<sgrid, KNT, 0, s>>>(p);
+        chain(kl_seg_kernel, sgrid, KNT, 0, s)(p);
         return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
     };
     if (L.n_ops > 0) {
@@ -494,7 +499,7 @@ int launch_kloc(const KlocLaunch& L, cudaStream_t s)
         const size_t smem = 4 * (size_t)((L.n_vars + 31) / 32);
         if (cudaFuncSetAttribute(kl_filter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
             return AMC_E_CUDA;
-        kl_bitmap_kernel<<<(unsigned)((L.n_vars + 255) / 256), 256, 0, s>>>(L.final_status, L.n_vars, bm);
+        chain(kl_bitmap_kernel, (unsigned)((L.n_vars + 255) / 256), 256, 0, s)(L.final_status, L.n_vars, bm);
         int32_t* cnt = reinterpret_cast<int32_t*>(w + lay.cnt);
         int64_t* off = reinterpret_cast<int64_t*>(w + lay.off);
         for (int64_t e0 = S; e0 < L.n_ops;) {
@@ -519,11 +524,11 @@ int launch_kloc(const KlocLaunch& L, cudaStream_t s)
                 return AMC_E_CUDA;
             const int64_t ns = (q.n + KSTRETCH - 1) / KSTRETCH;
             const int64_t fb = (ns + KFT / 32 - 1) / (KFT / 32), cb = (ns + 7) / 8;
-            kl_filter_kernel<<<(unsigned)(fb < n_sm ? fb : n_sm), KFT, smem, s>>>(q);
+            chain(kl_filter_kernel, (unsigned)(fb < n_sm ? fb : n_sm), KFT, smem, s)(q);
             if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
             int rc = dscan_exclusive(cnt, off, ns, w + lay.scan, s);
             if (rc) return rc;
-            kl_compact_kernel<<<(unsigned)(cb < 8 * n_sm ? cb : 8 * n_sm), 256, 0, s>>>(key[1], val[1], cnt, off, ns, key[0],
+            chain(kl_compact_kernel, (unsigned)(cb < 8 * n_sm ? cb : 8 * n_sm), 256, 0, s)(key[1], val[1], cnt, off, ns, key[0],
                                                                                      val[0]);
             if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
             rc = check(q.n, off + ns, w + lay.st);

@@ -64,6 +64,7 @@ struct OvParams {
 __global__ void ov_keys_kernel(const int32_t* __restrict__ start, const int32_t* __restrict__ len, int32_t A,
                                uint32_t* __restrict__ key, uint32_t* __restrict__ val, int* err)
 {
+    follow();
     const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= A) return;
     const int32_t s = start[a], l = len[a];
@@ -94,6 +95,7 @@ constexpr int OV_STEP = 4;
 template <bool FILL>
 __global__ void ov_sweep_kernel(const OvParams p)
 {
+    follow();
     const int64_t pos = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (pos >= p.A) return;
@@ -140,6 +142,7 @@ __global__ void ov_sweep_kernel(const OvParams p)
 __global__ void ov_total_kernel(const int64_t* __restrict__ off, int64_t NL, int64_t cap, int64_t* n_pairs, int* err,
                                 int* gate)
 {
+    follow();
     const int64_t t = off[NL];
     if (n_pairs) *n_pairs = t;
     const bool over = cap > 0 && t > cap;
@@ -151,12 +154,14 @@ __global__ void ov_total_kernel(const int64_t* __restrict__ off, int64_t NL, int
 // that was not written
 __global__ void ov_clear_kernel(int64_t* __restrict__ off, int64_t NL, const int* gate)
 {
+    follow();
     const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (*gate && a <= NL) off[a] = 0;
 }
 
 __global__ void ov_zero_kernel(int32_t* __restrict__ cnt, int64_t NL)
 {
+    follow();
     const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (a < NL) cnt[a] = 0;
 }
@@ -166,6 +171,7 @@ __global__ void ov_zero_kernel(int32_t* __restrict__ cnt, int64_t NL)
 __global__ void ov_copy_kernel(const uint32_t* __restrict__ other, const uint32_t* __restrict__ owner_list,
                                uint32_t* __restrict__ dst, const OvParams p, int64_t NL)
 {
+    follow();
     if (p.off[NL] > p.cap) return;
     const int64_t n = p.off[NL];
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -179,6 +185,7 @@ __global__ void ov_copy_kernel(const uint32_t* __restrict__ other, const uint32_
 template <bool FILL>
 __global__ void __launch_bounds__(256) ov_direct_kernel(const OvParams p, uint32_t* __restrict__ idx)
 {
+    follow();
     const int lane = threadIdx.x & 31;
     const int32_t a = (int32_t)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (a >= p.A) return;
@@ -284,18 +291,18 @@ int launch_overlaps(const OverlapBuild& O, cudaStream_t s)
     if (!O.arr_born && A <= OV_DIRECT) {
         int* gate = reinterpret_cast<int*>(w + L.gate);
         const unsigned wb = (unsigned)((A + 7) / 8);
-        ov_direct_kernel<false><<<wb, 256, 0, s>>>(p, nullptr);
+        chain(ov_direct_kernel<false>, wb, 256, 0, s)(p, nullptr);
         int rc = dscan_exclusive(p.cnt, O.ov_off, NL, w + L.scan, s);
         if (rc) return rc;
-        ov_total_kernel<<<1, 1, 0, s>>>(O.ov_off, NL, O.cap, O.n_pairs, O.err, gate);
+        chain(ov_total_kernel, 1, 1, 0, s)(O.ov_off, NL, O.cap, O.n_pairs, O.err, gate);
         if (O.cap > 0 && O.ov_idx) {
-            ov_direct_kernel<true><<<wb, 256, 0, s>>>(p, O.ov_idx);
-            ov_clear_kernel<<<lb, 256, 0, s>>>(O.ov_off, NL, gate);
+            chain(ov_direct_kernel<true>, wb, 256, 0, s)(p, O.ov_idx);
+            chain(ov_clear_kernel, lb, 256, 0, s)(O.ov_off, NL, gate);
         }
         return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
     }
-    ov_keys_kernel<<<ab, 256, 0, s>>>(O.arr_start, O.arr_len, A, k[0], v[0], O.err);
-    ov_zero_kernel<<<lb, 256, 0, s>>>(p.cnt, NL);
+    chain(ov_keys_kernel, ab, 256, 0, s)(O.arr_start, O.arr_len, A, k[0], v[0], O.err);
+    chain(ov_zero_kernel, lb, 256, 0, s)(p.cnt, NL);
     int passes = 0;
     // starts are < 2^31: 31 key bits
     int rc = launch_ss_radix(k, v, nullptr, A, INT32_MAX, w + L.sscr, nullptr, s, &passes);
@@ -303,18 +310,18 @@ int launch_overlaps(const OverlapBuild& O, cudaStream_t s)
     p.skey = k[passes & 1];
     p.sval = v[passes & 1];
     const unsigned wb = (unsigned)(((int64_t)A * 32 + 255) / 256);
-    ov_sweep_kernel<false><<<dim3(wb, OV_SPLIT), 256, 0, s>>>(p);
+    chain(ov_sweep_kernel<false>, dim3(wb, OV_SPLIT), 256, 0, s)(p);
     rc = dscan_exclusive(p.cnt, O.ov_off, NL, w + L.scan, s);
     if (rc) return rc;
     int* gate = reinterpret_cast<int*>(w + L.gate);
-    ov_total_kernel<<<1, 1, 0, s>>>(O.ov_off, NL, O.cap, O.n_pairs, O.err, gate);
+    chain(ov_total_kernel, 1, 1, 0, s)(O.ov_off, NL, O.cap, O.n_pairs, O.err, gate);
     if (O.cap <= 0 || !O.ov_idx) return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;   // count only
-    ov_zero_kernel<<<lb, 256, 0, s>>>(p.cnt, NL);
+    chain(ov_zero_kernel, lb, 256, 0, s)(p.cnt, NL);
     uint32_t* pk[2] = {reinterpret_cast<uint32_t*>(w + L.p0), reinterpret_cast<uint32_t*>(w + L.p1)};
     uint32_t* pv[2] = {reinterpret_cast<uint32_t*>(w + L.p2), reinterpret_cast<uint32_t*>(w + L.p3)};
     p.pkey = pk[0];
     p.pval = pv[0];
-    ov_sweep_kernel<true><<<dim3(wb, OV_SPLIT), 256, 0, s>>>(p);
+    chain(ov_sweep_kernel<true>, dim3(wb, OV_SPLIT), 256, 0, s)(p);
     // by other, then (stably) by owner list; the count is read on the device
     const int64_t* n_dev = O.ov_off + NL;
     rc = launch_ss_radix(pk, pv, n_dev, O.cap, A, w + L.pscr, gate, s, &passes);
@@ -329,9 +336,9 @@ int launch_overlaps(const OverlapBuild& O, cudaStream_t s)
     int dev = 0, n_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    ov_copy_kernel<<<(unsigned)(n_sm > 0 ? 4 * n_sm : 256), 256, 0, s>>>(v2[passes2 & 1], k2[passes2 & 1], O.ov_idx, p,
+    chain(ov_copy_kernel, (unsigned)(n_sm > 0 ? 4 * n_sm : 256), 256, 0, s)(v2[passes2 & 1], k2[passes2 & 1], O.ov_idx, p,
                                                                            NL);
-    ov_clear_kernel<<<lb, 256, 0, s>>>(O.ov_off, NL, gate);
+    chain(ov_clear_kernel, lb, 256, 0, s)(O.ov_off, NL, gate);
     return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
 }
 

@@ -90,6 +90,7 @@ __global__ void __launch_bounds__(SNT) ss_hist_kernel(const uint32_t* __restrict
                                                       int64_t cap, int shift, uint32_t* __restrict__ hist,
                                                       const int* gate)
 {
+    follow();
     __shared__ uint32_t cnt[SRAD];
     if (gated(gate)) return;
     const int64_t n = set_count(n_dev, cap);
@@ -115,6 +116,7 @@ __global__ void __launch_bounds__(SNT) ss_hist_kernel(const uint32_t* __restrict
 __global__ void __launch_bounds__(1024) ss_hscan_kernel(uint32_t* __restrict__ hist, uint32_t* __restrict__ dtot,
                                                         const int64_t* n_dev, int64_t cap, const int* gate)
 {
+    follow();
     __shared__ int tmp[1024 / 32 + 1];
     if (gated(gate)) return;
     const int64_t n = set_count(n_dev, cap);
@@ -155,6 +157,7 @@ __global__ void __launch_bounds__(SCT, 5) ss_scatter_kernel(const uint32_t* __re
                                                          const uint32_t* __restrict__ hist,
                                                          const uint32_t* __restrict__ dtot, const int* gate)
 {
+    follow();
     __shared__ __align__(16) uint32_t sk[ST];
     __shared__ __align__(16) uint32_t sv[ST];
     __shared__ uint32_t wcnt[SCW][SRAD];                    // per-warp digit counters, then their prefixes
@@ -357,6 +360,7 @@ __device__ __forceinline__ void thread_run(const SegParams& p, const SegTables& 
 //       tile's scan so that their latency overlaps it.
 __global__ void __launch_bounds__(SNT, 6) ss_red_kernel(const SegParams p)
 {
+    follow();
     __shared__ SegTables S;
     __shared__ uint32_t wtot[SNT / 32];
     if (gated(p.gate)) return;
@@ -379,6 +383,7 @@ constexpr int CNT = 1024;                  // threads of the carry CTA
 
 __global__ void __launch_bounds__(CNT) ss_carry_kernel(const SegParams p)
 {
+    follow();
     __shared__ uint8_t comp[MAX_ELEMS * MAX_ELEMS];
     __shared__ uint32_t wtot[CNT / 32];
     __shared__ uint8_t s_id;
@@ -417,6 +422,7 @@ __global__ void __launch_bounds__(CNT) ss_carry_kernel(const SegParams p)
 
 __global__ void __launch_bounds__(SNT, 4) ss_apply_kernel(const SegParams p)
 {
+    follow();
     __shared__ SegTables S;
     __shared__ uint32_t wtot[SNT / 32];
     if (gated(p.gate)) return;
@@ -550,6 +556,7 @@ __device__ __forceinline__ void forget(uint32_t* seen, uint32_t lv) { atomicAnd(
 
 __global__ void __launch_bounds__(BKW * 32, 1) ss_bucket_kernel(const BucketParams p)
 {
+    follow();
     extern __shared__ __align__(16) uint8_t rows[];        // [BKW][W], then seen bits [BKW][W / 32]
     __shared__ uint8_t comp[MAX_ELEMS * MAX_ELEMS];
     __shared__ uint8_t app[MAX_ELEMS * 8];
@@ -731,6 +738,7 @@ __global__ void ss_keys_kernel(const uint8_t* __restrict__ kind_side, const int3
                                int64_t n_after, int32_t n_vars, uint32_t* __restrict__ key,
                                uint32_t* __restrict__ val, uint8_t* __restrict__ step, int* err)
 {
+    follow();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const uint32_t ks = kind_side[i];
@@ -786,7 +794,7 @@ int launch_ss_keys(const uint8_t* kind_side, const int32_t* var, int64_t n, int6
     if (n <= 0) return AMC_OK;
     const int64_t blocks = (n + 255) / 256;
     const int grid = (int)(blocks < (int64_t)sm_count() * 8 ? blocks : (int64_t)sm_count() * 8);
-    ss_keys_kernel<<<grid, 256, 0, s>>>(kind_side, var, n, n_after, n_vars, key, val, step, err);
+    chain(ss_keys_kernel, grid, 256, 0, s)(kind_side, var, n, n_after, n_vars, key, val, step, err);
     return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
 }
 
@@ -807,9 +815,9 @@ int launch_ss_radix(uint32_t* const key[2], uint32_t* const val[2], const int64_
     for (int ps = 0; ps < passes; ++ps) {
         const int src = ps & 1;
         const int shift = ps * SDIG;
-        ss_hist_kernel<<<grid(8), SNT, 0, s>>>(key[src], n_dev, cap, shift, hist, gate);
-        ss_hscan_kernel<<<SRAD, 1024, 0, s>>>(hist, dtot, n_dev, cap, gate);
-        ss_scatter_kernel<<<grid(5), SCT, 0, s>>>(key[src], val[src], key[src ^ 1], val[src ^ 1], n_dev, cap, shift,
+        chain(ss_hist_kernel, grid(8), SNT, 0, s)(key[src], n_dev, cap, shift, hist, gate);
+        chain(ss_hscan_kernel, SRAD, 1024, 0, s)(hist, dtot, n_dev, cap, gate);
+        chain(ss_scatter_kernel, grid(5), SCT, 0, s)(key[src], val[src], key[src ^ 1], val[src ^ 1], n_dev, cap, shift,
                                                      hist, dtot, gate);
         if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
     }
@@ -848,9 +856,9 @@ int launch_sorted_check(const SortedCheck& C, cudaStream_t s)
     p.err = C.err;
     p.bm = C.bm;
     p.tab = host_tables();
-    ss_red_kernel<<<grid(6), SNT, 0, s>>>(p);
-    ss_carry_kernel<<<1, CNT, 0, s>>>(p);
-    ss_apply_kernel<<<grid(4), SNT, 0, s>>>(p);
+    chain(ss_red_kernel, grid(6), SNT, 0, s)(p);
+    chain(ss_carry_kernel, 1, CNT, 0, s)(p);
+    chain(ss_apply_kernel, grid(4), SNT, 0, s)(p);
     return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
 }
 
@@ -877,9 +885,9 @@ int launch_bucket_check(const SortedCheck& C, cudaStream_t s)
     uint8_t* w = static_cast<uint8_t*>(C.scratch);
     uint32_t* hist = reinterpret_cast<uint32_t*>(w);
     uint32_t* dtot = reinterpret_cast<uint32_t*>(w + align_up(4 * SRAD * (size_t)tiles, 256));
-    ss_hist_kernel<<<grid(8), SNT, 0, s>>>(C.key[0], C.n_dev, C.cap, 0, hist, C.gate);
-    ss_hscan_kernel<<<SRAD, 1024, 0, s>>>(hist, dtot, C.n_dev, C.cap, C.gate);
-    ss_scatter_kernel<<<grid(5), SCT, 0, s>>>(C.key[0], C.val[0], C.key[1], C.val[1], C.n_dev, C.cap, 0, hist,
+    chain(ss_hist_kernel, grid(8), SNT, 0, s)(C.key[0], C.n_dev, C.cap, 0, hist, C.gate);
+    chain(ss_hscan_kernel, SRAD, 1024, 0, s)(hist, dtot, C.n_dev, C.cap, C.gate);
+    chain(ss_scatter_kernel, grid(5), SCT, 0, s)(C.key[0], C.val[0], C.key[1], C.val[1], C.n_dev, C.cap, 0, hist,
                                               dtot, C.gate);
     BucketParams p;
     p.key = C.key[1];
@@ -898,7 +906,7 @@ int launch_bucket_check(const SortedCheck& C, cudaStream_t s)
     p.offset = C.offset;
     p.bm = C.bm;
     p.tab = host_tables();
-    ss_bucket_kernel<<<C.n_vars < SRAD ? C.n_vars : SRAD, BKW * 32, smem, s>>>(p);
+    chain(ss_bucket_kernel, C.n_vars < SRAD ? C.n_vars : SRAD, BKW * 32, smem, s)(p);
     return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
 }
 

@@ -179,6 +179,7 @@ TailLayout tail_layout(const TailShape& sh, int32_t n_vars, int64_t n_ops)
 // bit v: status of v is F
 __global__ void tail_bitmap_kernel(const uint8_t* __restrict__ st, int32_t n_vars, uint32_t* __restrict__ bm)
 {
+    follow();
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool f = v < n_vars && st[v] == ST_F;
     const uint32_t m = __ballot_sync(0xffffffffu, f);
@@ -213,6 +214,7 @@ struct FilterParams {
 template <int CHUNK>
 __global__ void __launch_bounds__(TF_THREADS, 1) tail_filter_kernel(const FilterParams q)
 {
+    follow();
     extern __shared__ __align__(16) uint32_t sbm[];
     for (int i = threadIdx.x; i < q.bm_words; i += TF_THREADS) sbm[i] = q.bm[i];
     __syncthreads();
@@ -360,6 +362,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) tail_filter_kernel(const Filter
 __global__ void __launch_bounds__(1024) tail_blocksum_kernel(const uint32_t* __restrict__ cnt, int n_chunks,
                                                              uint32_t* __restrict__ bsum)
 {
+    follow();
     __shared__ uint32_t ws[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = blockIdx.x * 1024 + threadIdx.x;
@@ -387,6 +390,7 @@ __global__ void __launch_bounds__(1024) tail_offsets_kernel(const uint32_t* __re
                                                             int64_t cap, uint32_t* __restrict__ coff,
                                                             int64_t* __restrict__ n_cand, int* ovf)
 {
+    follow();
     __shared__ unsigned long long rb[32], rt[32];
     __shared__ uint32_t wsum[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -459,6 +463,7 @@ __global__ void __launch_bounds__(256) tail_gather_kernel(const uint8_t* __restr
                                                           uint32_t* __restrict__ cpos, int G, int chunk, int slots,
                                                           const int* ovf)
 {
+    follow();
     if (*ovf) return;
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -503,6 +508,7 @@ __global__ void tail_post_kernel(const int* gate, const uint8_t* __restrict__ st
                                  const int32_t* __restrict__ fvff, int64_t* __restrict__ ff,
                                  const int64_t* __restrict__ fff, int64_t offset)
 {
+    follow();
     if (*gate == 0) return;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t n_words = ((int64_t)n_vars + 31) / 32 * 32;
@@ -635,7 +641,7 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
     // the stuck bitmap at the first epoch's start; later epochs add the
     // variables that become stuck (the bucket checks set their bits, the
     // fallback rebuilds it)
-    tail_bitmap_kernel<<<(unsigned)((L.n_vars + 255) / 256), 256, 0, s>>>(st[0], L.n_vars, bm);
+    chain(tail_bitmap_kernel, (unsigned)((L.n_vars + 255) / 256), 256, 0, s)(st[0], L.n_vars, bm);
 
     int cur = 0;
     for (int64_t e0 = sh.S; e0 < L.n_ops;) {
@@ -666,18 +672,18 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
         const int n_chunks = (int)chunks_of(n);
         const int fgrid = (int)min((int64_t)n_sm, ((int64_t)n_chunks + TF_THREADS / 32 - 1) / (TF_THREADS / 32));
         if (chunk == TF_CHUNK)
-            tail_filter_kernel<TF_CHUNK><<<fgrid, TF_THREADS, fsmem, s>>>(q);
+            chain(tail_filter_kernel<TF_CHUNK>, fgrid, TF_THREADS, fsmem, s)(q);
         else
-            tail_filter_kernel<TF_CHUNK_SHORT><<<fgrid, TF_THREADS, fsmem, s>>>(q);
+            chain(tail_filter_kernel<TF_CHUNK_SHORT>, fgrid, TF_THREADS, fsmem, s)(q);
         const int n_blocks = (n_chunks + 1023) / 1024;
         const int64_t C = cand_cap(n);
-        tail_blocksum_kernel<<<n_blocks, 1024, 0, s>>>(cnt, n_chunks, bsum);
-        tail_offsets_kernel<<<n_blocks, 1024, 0, s>>>(cnt, n_chunks, bsum, n_blocks, C, coff, ncand, ovf);
+        chain(tail_blocksum_kernel, n_blocks, 1024, 0, s)(cnt, n_chunks, bsum);
+        chain(tail_offsets_kernel, n_blocks, 1024, 0, s)(cnt, n_chunks, bsum, n_blocks, C, coff, ncand, ovf);
         int G = 1;                                   // chunks per gather warp: about 8,192 warps
         while (G < 32 && n_chunks / (2 * G) >= 8192) G *= 2;
         const int64_t groups = ((int64_t)n_chunks + G - 1) / G;
         const int ggrid = (int)min((int64_t)n_sm * 8, (groups + 7) / 8);
-        tail_gather_kernel<<<ggrid, 256, 0, s>>>(sks, svar, spos, cnt, coff, n_chunks, key0, val0, cpos, G, chunk, slots,
+        chain(tail_gather_kernel, ggrid, 256, 0, s)(sks, svar, spos, cnt, coff, n_chunks, key0, val0, cpos, G, chunk, slots,
                                                  ovf);
         if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
         // the candidates, at most C (count on the device), from the epoch's
@@ -724,7 +730,7 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
         F.profile = 0;
         rc = launch_scan_trace(F, s);
         if (rc) return rc;
-        tail_post_kernel<<<n_sm * 2, 256, 0, s>>>(ovf, fin, L.n_vars, bm, L.vff, fvff, L.first_fault, fff, e0);
+        chain(tail_post_kernel, n_sm * 2, 256, 0, s)(ovf, fin, L.n_vars, bm, L.vff, fvff, L.first_fault, fff, e0);
         if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
         cur ^= 1;
         e0 = e1;

@@ -1482,6 +1482,7 @@ __device__ __forceinline__ void issue_tile(const ScanParams& p, ScanSmem<KeyT, T
 template <typename KeyT, int T, int NT>
 __global__ void __launch_bounds__(NT, MAX_CTAS_PER_SM) scan_trace_kernel(const ScanParams p)
 {
+    follow();
     extern __shared__ __align__(128) uint8_t smem_raw[];
     // gated off: return before touching the tile counter or any other state
     // (a gated launch's set-up is gated the same way, so that state is stale)
@@ -1596,6 +1597,7 @@ __global__ void finalize_trace_kernel(int32_t* __restrict__ vff, const uint32_t*
                                       int32_t n_vars, uint8_t* __restrict__ final_status, const int* gate,
                                       int gate_on)
 {
+    follow();
     if (gate && ((*gate != 0) != (gate_on != 0))) return;     // gated off: the other launch writes
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n_vars; v += stride) {
@@ -1617,6 +1619,7 @@ __global__ void finalize_trace_kernel(int32_t* __restrict__ vff, const uint32_t*
 __global__ void seed_stuck_kernel(const uint8_t* __restrict__ init, int32_t n_vars, uint32_t* __restrict__ fbits,
                                   int fbits_words, const int* gate, int gate_on)
 {
+    follow();
     if (gate && ((*gate != 0) != (gate_on != 0))) return;
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool f = v < n_vars && init[v] == ST_F;
@@ -1638,6 +1641,7 @@ __global__ void gated_init_kernel(const int* gate, int gate_on, uint32_t* __rest
                                   int64_t f_words, const uint8_t* __restrict__ init,
                                   uint32_t* __restrict__ tile_counter)
 {
+    follow();
     if ((*gate != 0) != (gate_on != 0)) return;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1701,7 +1705,7 @@ int launch_kernel(ScanParams p, const ScanLaunch& L, cudaStream_t s)
     if (grid > p.n_tiles) grid = p.n_tiles;
     if (L.max_ctas > 0 && grid > L.max_ctas) grid = L.max_ctas;
     if (L.profile & 1) profile_begin(s);
-    scan_trace_kernel<KeyT, TILE, THREADS><<<grid, THREADS, smem, s>>>(p);
+    chain(scan_trace_kernel<KeyT, TILE, THREADS>, grid, THREADS, smem, s)(p);
     if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
     if (L.profile & 2) profile_end(s);
     return AMC_OK;
@@ -1851,7 +1855,7 @@ int launch_scan_trace(const ScanLaunch& L, cudaStream_t s)
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dv);
         const int64_t cap = n_sm > 0 ? 4 * (int64_t)n_sm : 4096;       // grid-stride; a gated-off launch is cheap
         const int nb = (int)((nw + 255) / 256 < cap ? (nw + 255) / 256 : cap);
-        gated_init_kernel<<<nb > 0 ? nb : 1, 256, 0, s>>>(L.gate, L.gate_on, p.head, L.vff, L.n_vars,
+        chain(gated_init_kernel, nb > 0 ? nb : 1, 256, 0, s)(L.gate, L.gate_on, p.head, L.vff, L.n_vars,
                                                           L.first_fault, p.regbits, L.n_ops > 0 ? regbytes / 4 : 0,
                                                           p.fbits, L.n_ops > 0 ? p.fbits_words : 0, L.init,
                                                           p.tile_counter);
@@ -1867,7 +1871,7 @@ int launch_scan_trace(const ScanLaunch& L, cudaStream_t s)
             if (fbytes && cudaMemsetAsync(p.fbits, 0, fbytes, s) != cudaSuccess) return AMC_E_CUDA;
         }
         if (L.init && L.n_vars > 0 && !L.gate) {
-            seed_stuck_kernel<<<(unsigned)((L.n_vars + 255) / 256), 256, 0, s>>>(L.init, L.n_vars, p.fbits,
+            chain(seed_stuck_kernel, (unsigned)((L.n_vars + 255) / 256), 256, 0, s)(L.init, L.n_vars, p.fbits,
                                                                                 p.fbits_words, L.gate, L.gate_on);
             if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
         }
@@ -1884,7 +1888,7 @@ int launch_scan_trace(const ScanLaunch& L, cudaStream_t s)
         const int64_t cap = n_sm > 0 ? 8 * (int64_t)n_sm : 4096;       // grid-stride
         const int nb = (int)((L.n_vars + 255) / 256 < cap ? (L.n_vars + 255) / 256 : cap);
         if (nb > 0) {
-            finalize_trace_kernel<<<nb, 256, 0, s>>>(L.vff, p.head, p.node_status, L.init, L.n_vars,
+            chain(finalize_trace_kernel, nb, 256, 0, s)(L.vff, p.head, p.node_status, L.init, L.n_vars,
                                                      L.final_status, L.gate, L.gate_on);
             if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
         }
