@@ -35,8 +35,14 @@ constexpr int TF_THREADS = 1024;          // filter CTA: one per SM (the bitmap 
 constexpr int TF_CHUNK = 4096;            // ops per warp chunk in epochs of 2^27 ops or more,
 constexpr int TF_CHUNK_SHORT = 1024;      // in shorter epochs (more warps busy)
 constexpr int64_t TF_LONG_CHUNKS_FROM = (int64_t)1 << 27;
-constexpr int TF_SLOT_DIV = 4;            // candidate slots per chunk: a quarter (more: the epoch falls back)
-constexpr int CAND_DIV = 4;               // candidate capacity: epoch ops / 4 (more: falls back)
+// Candidate slots per chunk, and candidates per epoch: a quarter of the ops, half
+// in epochs of at most 2^24 ops (more: the epoch falls back).  The early epochs
+// have the most: a mostly right trace of 150 M ops over a million variables had
+// 24 % candidates in its first epoch (6.3 M ops) and over a quarter in 826 of its
+// 6,144 chunks, and fell back: 1,581 us, 1,150 with half.  Half of a short epoch costs
+// no scratch where a longer one follows.  Later epochs have 16, 9 and 4 %.
+constexpr int TF_SLOT_DIV = 4;
+constexpr int64_t TF_HALF_TO = (int64_t)1 << 24;
 constexpr int64_t CAND_MAX = (int64_t)1 << 27;   // and at most 2^27 (set index << 4 fits 32 bits)
 constexpr int TF_PER = 16;                // ops per lane and step
 constexpr int TAIL_MIN_VARS = 16385;      // fewer variables take the reduce / carry / apply path
@@ -87,8 +93,8 @@ bool tail_shape(int64_t n_ops, int32_t n_vars, bool guarded, TailShape& sh, int 
 // ops per filter chunk of an epoch of n ops
 int chunk_for(int64_t n) { return n < TF_LONG_CHUNKS_FROM ? TF_CHUNK_SHORT : TF_CHUNK; }
 int64_t chunks_of(int64_t n) { return (n + chunk_for(n) - 1) / chunk_for(n); }
-// candidate slots per chunk: a quarter of it
-int slots_for(int64_t n) { return chunk_for(n) / TF_SLOT_DIV; }
+int slot_div(int64_t n) { return n <= TF_HALF_TO ? TF_SLOT_DIV / 2 : TF_SLOT_DIV; }
+int slots_for(int64_t n) { return chunk_for(n) / slot_div(n); }
 
 int64_t epoch_end(const TailShape& sh, int64_t e0, int64_t n_ops)
 {
@@ -109,7 +115,7 @@ int64_t longest_epoch(const TailShape& sh, int64_t n_ops)
 // candidate capacity of an epoch of E ops
 int64_t cand_cap(int64_t E)
 {
-    int64_t C = (E + CAND_DIV - 1) / CAND_DIV;
+    int64_t C = (E + slot_div(E) - 1) / slot_div(E);
     C = (C + TF_CHUNK - 1) / TF_CHUNK * TF_CHUNK;
     return C < CAND_MAX ? C : CAND_MAX;
 }
@@ -137,8 +143,9 @@ TailLayout tail_layout(const TailShape& sh, int32_t n_vars, int64_t n_ops)
         if ((size_t)chunks_of(n) > n_chunks) n_chunks = (size_t)chunks_of(n);
         if ((size_t)(chunks_of(n) * slots_for(n)) > n_slots) n_slots = (size_t)(chunks_of(n) * slots_for(n));
     }
-    const int64_t C = cand_cap(Emax);
-    t.K = C > sh.S ? C : sh.S;
+    t.K = sh.S;
+    for (int64_t e0 = sh.S; e0 < n_ops; e0 = epoch_end(sh, e0, n_ops))
+        if (const int64_t C = cand_cap(epoch_end(sh, e0, n_ops) - e0); C > t.K) t.K = C;
     const size_t K = (size_t)t.K;
     size_t o = 0;
     auto take = [&](size_t b) { const size_t at = o; o += align_up(b, 256); return at; };
@@ -195,13 +202,14 @@ struct FilterParams {
     const uint32_t* bm;         // stuck bitmap at the epoch's start
     int bm_words;
     uint8_t* step;              // the epoch's outputs
-    uint8_t* sks;               // candidate slots: a quarter of the chunk
+    uint8_t* sks;               // candidate slots, `slots` per chunk
     int32_t* svar;
     uint16_t* spos;             // position within the chunk
     uint32_t* cnt;              // candidates per chunk
     int* ovf;                   // set when a chunk has more candidates than slots
     int* err;
     int bulk_ok;
+    int slots;
 };
 
 // Each warp takes chunks of CHUNK ops in steps of 32 x 16 (lane L: ops
@@ -336,13 +344,13 @@ __global__ void __launch_bounds__(TF_THREADS, 1) tail_filter_kernel(const Filter
                 pre += __popc(bal & lt) << bit;
                 wtot += __popc(bal) << bit;
             }
-            if (wcount + wtot > CHUNK / TF_SLOT_DIV) {
+            if (wcount + wtot > q.slots) {
                 // more candidates than slots: the epoch is rechecked whole
                 if (lane == 0) atomicExch(q.ovf, 1);
                 full = true;
                 continue;
             }
-            int64_t idx = c * (CHUNK / TF_SLOT_DIV) + wcount + pre;
+            int64_t idx = c * q.slots + wcount + pre;
 #pragma unroll
             for (int u = 0; u < TF_PER; ++u) {
                 if (liveMask & (1u << u)) {
@@ -666,6 +674,7 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
         q.spos = spos;
         q.cnt = cnt;
         q.ovf = ovf;
+        q.slots = slots;
         q.err = L.err;
         q.bulk_ok = ((uintptr_t)q.kind_side % 16 == 0) && ((uintptr_t)q.var % 16 == 0) &&
                     ((uintptr_t)q.step % 16 == 0);
