@@ -207,6 +207,22 @@ __device__ __forceinline__ int block_excl_sum(int x, int* tmp, int* total)
 
 __host__ __device__ constexpr size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// Lanes (of those with ok) that hold the same v as this lane, when the lanes that
+// lost their place to another with the same v are known: one round per value that
+// several lanes hold, where match.any takes one per value.  All lanes call it.
+__device__ __forceinline__ uint32_t lanes_with_same(uint32_t v, bool ok, bool lost)
+{
+    uint32_t peers = 1u << (threadIdx.x & 31);
+    for (uint32_t rest = __ballot_sync(0xffffffffu, lost); rest;) {
+        const uint32_t x = __shfl_sync(0xffffffffu, v, __ffs(rest) - 1);
+        const bool same = ok && v == x;
+        const uint32_t m = __ballot_sync(0xffffffffu, same);
+        if (same) peers = m;
+        rest &= ~m;
+    }
+    return peers;
+}
+
 // Kernels of one call follow each other on its stream: chain(kernel, grid, block,
 // shared bytes, stream)(arguments...) lets a kernel's CTAs be set up while the
 // last ones of the kernel before it still run (programmatic dependent launch).

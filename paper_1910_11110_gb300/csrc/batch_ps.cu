@@ -425,7 +425,8 @@ __device__ void run_small(const PsParams& p, int64_t prog, PsWarp& S, const PsTa
                 step[wb + lane] = 0;
             }
             __syncwarp();
-            const bool dup = __any_sync(0xffffffffu, valid && S.tag[pl] != lane);
+            const bool lost = valid && S.tag[pl] != lane;
+            const bool dup = __any_sync(0xffffffffu, lost);
             if (!dup) {
                 if (valid) {
                     const uint32_t j = J[pl];
@@ -436,7 +437,7 @@ __device__ void run_small(const PsParams& p, int64_t prog, PsWarp& S, const PsTa
                 }
             } else {
                 S.ops[lane] = (uint8_t)o;
-                const uint32_t peers = __match_any_sync(0xffffffffu, valid ? (uint32_t)pl : 0x80000000u | lane);
+                const uint32_t peers = lanes_with_same((uint32_t)pl, valid, lost);
                 __syncwarp();
                 if (valid && (peers & lt) == 0) {
                     uint32_t j = J[pl];

@@ -504,15 +504,21 @@ __global__ void __launch_bounds__(SNT, 4) ss_apply_kernel(const SegParams p)
 //   (a) warp w folds its stretch of the bucket, 32 pairs at a time, into one
 //       function per variable of the bucket (a row of ceil(n_vars / 128)
 //       bytes in shared memory, indexed by v / 128): when the batch's
-//       variables are distinct (a bit per variable in shared memory tells)
-//       each lane composes its own, else lanes with the same variable are
-//       grouped (match.any) and the group's first lane composes them in order;
+//       variables are distinct (each lane leaves its number in its variable's
+//       byte and reads it back) each lane composes its own, else lanes with the
+//       same variable are grouped and the group's first lane composes them in
+//       order;
 //   (b) a thread per variable carries the entry status through the warps'
 //       functions: every stretch's entry statuses, and the final status (and
 //       stuck bit) of a variable whose status changed;
 //   (c) each warp re-runs its stretch from those entry statuses, writing the
 //       statuses that are not F (the caller wrote F everywhere) and the first
 //       faults.
+// What bounds it: 16 warps an SM, each waiting on its own chain of shared-memory
+// look-ups (about 16 us a set, 23 us a million pairs).  Telling equal variables by
+// a bit each in shared memory (two atomics a pair), loading the start statuses in
+// the carry, one variable after another: 1,150 us for 150 M mostly right ops,
+// 1,128 this way.  20 and 24 warps (more rows to carry through) were slower, and 8.
 constexpr int BKW = 16;                   // warps of a bucket CTA
 constexpr int BK_MAX_W = 8192;            // variables per bucket (n_vars <= 2^20): 128 KB of rows
 constexpr int BKU = 16;                   // batches of 32 pairs loaded at once
@@ -543,21 +549,10 @@ struct BucketParams {
     Tables tab;
 };
 
-// Duplicate test of a batch without match.any (slow on this part): each lane
-// sets its variable's bit in the warp's bitmap; a bit already set means that
-// an earlier lane of the batch has the same variable.  The bits are cleared
-// after the batch.
-__device__ __forceinline__ bool seen_before(uint32_t* seen, uint32_t lv)
-{
-    const uint32_t bit = 1u << (lv & 31);
-    return (atomicOr(seen + (lv >> 5), bit) & bit) != 0;
-}
-__device__ __forceinline__ void forget(uint32_t* seen, uint32_t lv) { atomicAnd(seen + (lv >> 5), ~(1u << (lv & 31))); }
-
 __global__ void __launch_bounds__(BKW * 32, 1) ss_bucket_kernel(const BucketParams p)
 {
     follow();
-    extern __shared__ __align__(16) uint8_t rows[];        // [BKW][W], then seen bits [BKW][W / 32]
+    extern __shared__ __align__(16) uint8_t rows[];        // [BKW][W], then the bucket's start statuses [W]
     __shared__ uint8_t comp[MAX_ELEMS * MAX_ELEMS];
     __shared__ uint8_t app[MAX_ELEMS * 8];
     __shared__ uint8_t elem[16];
@@ -581,10 +576,7 @@ __global__ void __launch_bounds__(BKW * 32, 1) ss_bucket_kernel(const BucketPara
     const uint32_t ID = p.tab.identity;
     const int W = bucket_width(p.n_vars);
     const int64_t n = set_count(p.n_dev, p.cap);
-    uint32_t* const seen_all = reinterpret_cast<uint32_t*>(rows + (size_t)BKW * W);
-    const int WS = (W + 31) >> 5;
-    uint32_t* const seen = seen_all + w * WS;             // this warp's bits
-    for (int i = tid; i < BKW * WS; i += BKW * 32) seen_all[i] = 0;
+    uint8_t* const first = rows + (size_t)BKW * W;
     __syncthreads();
     for (int b = blockIdx.x; b < SRAD; b += gridDim.x) {
         const int nv = (int)(((int64_t)p.n_vars - b + SRAD - 1) / SRAD);   // ids b, b + 128, ... below n_vars
@@ -595,6 +587,8 @@ __global__ void __launch_bounds__(BKW * 32, 1) ss_bucket_kernel(const BucketPara
         uint8_t* row = rows + (size_t)w * W;
         // rows start as "absent" (no pair of the variable in the stretch yet)
         for (int v = lane; v < W / 16; v += 32) reinterpret_cast<uint4*>(row)[v] = make_uint4(~0u, ~0u, ~0u, ~0u);
+        for (int lv = tid; lv < nv; lv += BKW * 32)
+            first[lv] = p.init ? (uint8_t)(p.init[(int64_t)lv * SRAD + b] & 7u) : (uint8_t)AMC_ST_VI;
         __syncwarp();
         // (a) fold the stretch per variable; BKU batches of 32 pairs are
         // loaded at once (their loads overlap), then folded one by one
@@ -612,24 +606,24 @@ __global__ void __launch_bounds__(BKW * 32, 1) ss_bucket_kernel(const BucketPara
                 const uint32_t lv = kk[u];
                 const bool ok = lv != 0xFFFFFFFFu;
                 const uint32_t m = ok ? elem[vv[u] & 15u] : ID;
-                if (!__ballot_sync(0xffffffffu, ok && seen_before(seen, lv))) {
+                const uint32_t r0 = ok ? row[lv] : ID;
+                __syncwarp();
+                if (ok) row[lv] = (uint8_t)lane;
+                __syncwarp();
+                const bool lost = ok && row[lv] != lane;
+                if (!__any_sync(0xffffffffu, lost)) {
                     // every variable once in the batch: each lane composes alone
-                    if (ok) {
-                        const uint32_t r = row[lv];
-                        row[lv] = r == BK_ABSENT ? (uint8_t)m : comp[r * MAX_ELEMS + m];
-                    }
+                    if (ok) row[lv] = r0 == BK_ABSENT ? (uint8_t)m : comp[r0 * MAX_ELEMS + m];
                 } else {
                     mb[w][lane] = (uint8_t)m;
-                    const uint32_t peers = __match_any_sync(0xffffffffu, lv);
+                    const uint32_t peers = lanes_with_same(lv, ok, lost);
                     __syncwarp();
                     if (ok && lane == __ffs(peers) - 1) {
-                        uint32_t acc = row[lv];
-                        if (acc == BK_ABSENT) acc = ID;
+                        uint32_t acc = r0 == BK_ABSENT ? ID : r0;
                         for (uint32_t r = peers; r; r &= r - 1) acc = comp[acc * MAX_ELEMS + mb[w][__ffs(r) - 1]];
                         row[lv] = (uint8_t)acc;
                     }
                 }
-                if (ok) forget(seen, lv);
                 __syncwarp();
             }
         }
@@ -647,23 +641,28 @@ __global__ void __launch_bounds__(BKW * 32, 1) ss_bucket_kernel(const BucketPara
                 all &= e4[k];
             }
             if (all == ~0u) continue;
+            // (beyond nv: no pairs, any status)
+            const uint32_t s0 = reinterpret_cast<const uint32_t*>(first)[l4];
+            uint32_t st[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) st[j] = (s0 >> (8 * j)) & 7u;
+#pragma unroll
+            for (int k = 0; k < BKW; ++k) {
+                reinterpret_cast<uint32_t*>(rows + (size_t)k * W)[l4] = st[0] | st[1] << 8 | st[2] << 16 | st[3] << 24;
+                if (e4[k] == ~0u) continue;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint32_t e = (e4[k] >> (8 * j)) & 0xFFu;
+                    if (e != BK_ABSENT) st[j] = app[e * 8 + st[j]];
+                }
+            }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int lv = 4 * l4 + j;
-                if (lv >= nv) break;
+                if (lv >= nv || st[j] == ((s0 >> (8 * j)) & 7u)) continue;
                 const int64_t v = (int64_t)lv * SRAD + b;
-                const uint32_t s0 = p.init ? (uint32_t)(p.init[v] & 7u) : (uint32_t)AMC_ST_VI;
-                uint32_t st = s0;
-#pragma unroll
-                for (int k = 0; k < BKW; ++k) {
-                    const uint32_t e = (e4[k] >> (8 * j)) & 0xFFu;
-                    rows[(size_t)k * W + lv] = (uint8_t)st;
-                    if (e != BK_ABSENT) st = app[e * 8 + st];
-                }
-                if (st != s0) {
-                    p.fin[v] = (uint8_t)st;
-                    if (p.bm && st == ST_F) atomicOr(p.bm + (v >> 5), 1u << (v & 31));
-                }
+                p.fin[v] = (uint8_t)st[j];
+                if (p.bm && st[j] == ST_F) atomicOr(p.bm + (v >> 5), 1u << (v & 31));
             }
         }
         __syncthreads();
@@ -688,17 +687,18 @@ __global__ void __launch_bounds__(BKW * 32, 1) ss_bucket_kernel(const BucketPara
                 const uint32_t posi = pp[u];
                 // pre / post: the variable's status before / after the pair
                 uint32_t pre = 0, post = 0;
-                if (!__ballot_sync(0xffffffffu, ok && seen_before(seen, lv))) {
-                    if (ok) {
-                        pre = row[lv];
-                        post = app[m * 8 + pre];
-                        row[lv] = (uint8_t)post;
-                    }
+                const uint32_t cur = ok ? row[lv] : 0u;
+                __syncwarp();
+                if (ok) row[lv] = (uint8_t)lane;
+                __syncwarp();
+                const bool lost = ok && row[lv] != lane;
+                if (!__any_sync(0xffffffffu, lost)) {
+                    pre = cur;
+                    post = app[m * 8 + pre];
+                    if (ok) row[lv] = (uint8_t)post;
                 } else {
                     mb[w][lane] = (uint8_t)m;
-                    const uint32_t peers = __match_any_sync(0xffffffffu, lv);
-                    __syncwarp();
-                    const uint32_t cur = ok ? row[lv] : 0u;
+                    const uint32_t peers = lanes_with_same(lv, ok, lost);
                     __syncwarp();
                     if (ok) {
                         uint32_t acc = ID;
@@ -709,7 +709,6 @@ __global__ void __launch_bounds__(BKW * 32, 1) ss_bucket_kernel(const BucketPara
                     }
                 }
                 if (ok) {
-                    forget(seen, lv);
                     if (post != ST_F) {
                         p.step[posi] = (uint8_t)post;
                     } else if (pre != ST_F) {
@@ -869,7 +868,7 @@ int launch_bucket_check(const SortedCheck& C, cudaStream_t s)
     if (C.cap <= 0) return AMC_OK;
     if (C.cap > ((int64_t)1 << 28) || !C.pos || !bucket_check_ok(C.n_vars)) return AMC_E_INVALID;
     const int W = bucket_width(C.n_vars);
-    const size_t smem = (size_t)BKW * W + (size_t)BKW * 4 * ((W + 31) / 32);
+    const size_t smem = (size_t)(BKW + 1) * W;
     static size_t attr_set[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
