@@ -732,13 +732,23 @@ __global__ void __launch_bounds__(BKW * 32, 1) ss_bucket_kernel(const BucketPara
 
 // Raw ops [0, n) as pairs: checked like the filter checks them (bad bytes,
 // ids out of range, GT not followed by its EN), F written at every position,
-// pairs (id, i << 4 | code) with bad ids replaced by 0.
+// pairs (id, i << 4 | code) with bad ids replaced by 0.  The check's start state
+// with them: no first faults, the variables' statuses, no overflow.
 __global__ void ss_keys_kernel(const uint8_t* __restrict__ kind_side, const int32_t* __restrict__ var, int64_t n,
                                int64_t n_after, int32_t n_vars, uint32_t* __restrict__ key,
-                               uint32_t* __restrict__ val, uint8_t* __restrict__ step, int* err)
+                               uint32_t* __restrict__ val, uint8_t* __restrict__ step, const SortedStart z, int* err)
 {
     follow();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (first == 0) {
+        *z.ff = -1;
+        *z.gate = 0;
+    }
+    for (int64_t v = first; v < n_vars; v += stride) {
+        z.vff[v] = -1;
+        z.status[v] = z.init ? z.init[v] : (uint8_t)AMC_ST_VI;
+    }
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const uint32_t ks = kind_side[i];
         const int32_t v = var[i];
@@ -788,12 +798,12 @@ size_t sorted_check_scratch_bytes(int64_t cap)
 }
 
 int launch_ss_keys(const uint8_t* kind_side, const int32_t* var, int64_t n, int64_t n_after, int32_t n_vars,
-                   uint32_t* key, uint32_t* val, uint8_t* step, int* err, cudaStream_t s)
+                   uint32_t* key, uint32_t* val, uint8_t* step, const SortedStart& z, int* err, cudaStream_t s)
 {
     if (n <= 0) return AMC_OK;
     const int64_t blocks = (n + 255) / 256;
     const int grid = (int)(blocks < (int64_t)sm_count() * 8 ? blocks : (int64_t)sm_count() * 8);
-    chain(ss_keys_kernel, grid, 256, 0, s)(kind_side, var, n, n_after, n_vars, key, val, step, err);
+    chain(ss_keys_kernel, grid, 256, 0, s)(kind_side, var, n, n_after, n_vars, key, val, step, z, err);
     return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
 }
 

@@ -156,7 +156,7 @@ TailLayout tail_layout(const TailShape& sh, int32_t n_vars, int64_t n_ops)
     t.off = take(4 * n_chunks);
     t.coff = take(4 * n_chunks);
     t.ncand = take(8);
-    t.ovf = take(4);
+    t.ovf = take(8);
     t.fvff = take(4 * (size_t)n_vars);
     t.fff = take(8);
     t.region = o;
@@ -511,12 +511,14 @@ __global__ void __launch_bounds__(256) tail_gather_kernel(const uint8_t* __restr
 // After an epoch's fallback scan (gated on by its overflow flag): the scan's
 // first faults folded into the trace's, the stuck bitmap rebuilt from the
 // statuses the scan wrote.
-__global__ void tail_post_kernel(const int* gate, const uint8_t* __restrict__ st, int32_t n_vars,
+__global__ void tail_post_kernel(const int* gate, int* next_gate, const uint8_t* __restrict__ fst,
+                                 uint8_t* __restrict__ st, int32_t n_vars,
                                  uint32_t* __restrict__ bm, int32_t* __restrict__ vff,
                                  const int32_t* __restrict__ fvff, int64_t* __restrict__ ff,
                                  const int64_t* __restrict__ fff, int64_t offset)
 {
     follow();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *next_gate = 0;
     if (*gate == 0) return;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t n_words = ((int64_t)n_vars + 31) / 32 * 32;
@@ -524,7 +526,8 @@ __global__ void tail_post_kernel(const int* gate, const uint8_t* __restrict__ st
         bool f = false;
         if (v < n_vars) {
             if (vff[v] == -1 && fvff[v] != -1) vff[v] = (int32_t)(fvff[v] + offset);
-            f = st[v] == ST_F;
+            st[v] = fst[v];
+            f = fst[v] == ST_F;
         }
         const uint32_t m = __ballot_sync(0xffffffffu, f);
         if ((threadIdx.x & 31) == 0) bm[v >> 5] = m;
@@ -580,13 +583,16 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
     if (!tail_shape(L.n_ops, L.n_vars, false, sh, L.tail)) return AMC_E_INVALID;
     const TailLayout lay = tail_layout(sh, L.n_vars, L.n_ops);
     uint8_t* w = static_cast<uint8_t*>(L.workspace);
-    uint8_t* st[2] = {w + lay.st0, w + lay.st1};
+    // the statuses as the trace goes on, where they are wanted in the end; a
+    // fallback's final ones
+    uint8_t* st = L.final_status ? L.final_status : w + lay.st0;
+    uint8_t* fst = w + lay.st1;
     uint32_t* bm = reinterpret_cast<uint32_t*>(w + lay.bm);
     uint32_t* cnt = reinterpret_cast<uint32_t*>(w + lay.cnt);
     uint32_t* bsum = reinterpret_cast<uint32_t*>(w + lay.off);    // candidates per 1024 chunks
     uint32_t* coff = reinterpret_cast<uint32_t*>(w + lay.coff);   // first candidate of each chunk
     int64_t* ncand = reinterpret_cast<int64_t*>(w + lay.ncand);
-    int* ovf = reinterpret_cast<int*>(w + lay.ovf);
+    int* ovf = reinterpret_cast<int*>(w + lay.ovf);            // two words, in turn: an epoch's end clears the next one's
     int32_t* fvff = reinterpret_cast<int32_t*>(w + lay.fvff);
     int64_t* fff = reinterpret_cast<int64_t*>(w + lay.fff);
     uint8_t* reg = w + lay.region;
@@ -619,16 +625,9 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
     if (L.profile & 1) profile_begin(s);
 
     // first part: ops [0, S) checked by sorting them by variable, from the
-    // initial statuses; final statuses to st[0]
-    if (cudaMemsetAsync(L.vff, 0xFF, 4 * (size_t)L.n_vars, s) != cudaSuccess) return AMC_E_CUDA;
-    if (cudaMemsetAsync(L.first_fault, 0xFF, 8, s) != cudaSuccess) return AMC_E_CUDA;
-    if (L.init) {
-        if (cudaMemcpyAsync(st[0], L.init, (size_t)L.n_vars, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-            return AMC_E_CUDA;
-    } else if (cudaMemsetAsync(st[0], AMC_ST_VI, (size_t)L.n_vars, s) != cudaSuccess) {
-        return AMC_E_CUDA;
-    }
-    int rc = launch_ss_keys(L.kind_side, L.var, sh.S, L.n_ops, L.n_vars, key0, val0, L.step, L.err, s);
+    // initial statuses; final statuses to st
+    const SortedStart z = {L.vff, L.first_fault, st, L.init, ovf};
+    int rc = launch_ss_keys(L.kind_side, L.var, sh.S, L.n_ops, L.n_vars, key0, val0, L.step, z, L.err, s);
     if (rc) return rc;
     SortedCheck A;
     A.key[0] = key0;
@@ -639,7 +638,7 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
     A.n_vars = L.n_vars;
     A.init = L.init;
     A.step = L.step;
-    A.fin = st[0];
+    A.fin = st;
     A.vff = L.vff;
     A.ff = L.first_fault;
     A.scratch = scratch;
@@ -649,15 +648,13 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
     // the stuck bitmap at the first epoch's start; later epochs add the
     // variables that become stuck (the bucket checks set their bits, the
     // fallback rebuilds it)
-    chain(tail_bitmap_kernel, (unsigned)((L.n_vars + 255) / 256), 256, 0, s)(st[0], L.n_vars, bm);
+    chain(tail_bitmap_kernel, (unsigned)((L.n_vars + 255) / 256), 256, 0, s)(st, L.n_vars, bm);
 
     int cur = 0;
-    for (int64_t e0 = sh.S; e0 < L.n_ops;) {
+    for (int64_t e0 = sh.S; e0 < L.n_ops; cur ^= 1) {
+        int* const gate = ovf + cur;
         const int64_t e1 = epoch_end(sh, e0, L.n_ops);
         const int64_t n = e1 - e0;
-        const bool last = e1 >= L.n_ops;
-        uint8_t* fin = (last && L.final_status) ? L.final_status : st[cur ^ 1];
-        if (cudaMemsetAsync(ovf, 0, sizeof(int), s) != cudaSuccess) return AMC_E_CUDA;
         const int chunk = chunk_for(n);
         const int slots = slots_for(n);
         FilterParams q;
@@ -673,7 +670,7 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
         q.svar = svar;
         q.spos = spos;
         q.cnt = cnt;
-        q.ovf = ovf;
+        q.ovf = gate;
         q.slots = slots;
         q.err = L.err;
         q.bulk_ok = ((uintptr_t)q.kind_side % 16 == 0) && ((uintptr_t)q.var % 16 == 0) &&
@@ -687,19 +684,18 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
         const int n_blocks = (n_chunks + 1023) / 1024;
         const int64_t C = cand_cap(n);
         chain(tail_blocksum_kernel, n_blocks, 1024, 0, s)(cnt, n_chunks, bsum);
-        chain(tail_offsets_kernel, n_blocks, 1024, 0, s)(cnt, n_chunks, bsum, n_blocks, C, coff, ncand, ovf);
+        chain(tail_offsets_kernel, n_blocks, 1024, 0, s)(cnt, n_chunks, bsum, n_blocks, C, coff, ncand, gate);
         int G = 1;                                   // chunks per gather warp: about 8,192 warps
         while (G < 32 && n_chunks / (2 * G) >= 8192) G *= 2;
         const int64_t groups = ((int64_t)n_chunks + G - 1) / G;
         const int ggrid = (int)min((int64_t)n_sm * 8, (groups + 7) / 8);
         chain(tail_gather_kernel, ggrid, 256, 0, s)(sks, svar, spos, cnt, coff, n_chunks, key0, val0, cpos, G, chunk, slots,
-                                                 ovf);
+                                                 gate);
         if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
         // the candidates, at most C (count on the device), from the epoch's
-        // start statuses, checked per bucket of ids (final statuses written
-        // where they change); gated off when they overflowed
-        if (cudaMemcpyAsync(fin, st[cur], (size_t)L.n_vars, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-            return AMC_E_CUDA;
+        // start statuses, checked per bucket of ids (a bucket's statuses are read
+        // and, where they change, written by its CTA); gated off when they
+        // overflowed
         SortedCheck K;
         K.key[0] = key0;
         K.key[1] = key1;
@@ -708,11 +704,11 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
         K.pos = cpos;
         K.n_dev = ncand;
         K.cap = C;
-        K.gate = ovf;
+        K.gate = gate;
         K.n_vars = L.n_vars;
-        K.init = st[cur];
+        K.init = st;
         K.step = L.step + e0;
-        K.fin = fin;
+        K.fin = st;
         K.vff = L.vff;
         K.ff = L.first_fault;
         K.offset = e0;
@@ -727,11 +723,11 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
         F.kind_side = L.kind_side + e0;
         F.var = L.var + e0;
         F.n_ops = n;
-        F.gate = ovf;
+        F.gate = gate;
         F.gate_on = 1;
-        F.init = st[cur];
+        F.init = st;
         F.step = L.step + e0;
-        F.final_status = fin;
+        F.final_status = fst;
         F.vff = fvff;
         F.first_fault = fff;
         F.workspace = reg;
@@ -739,9 +735,9 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
         F.profile = 0;
         rc = launch_scan_trace(F, s);
         if (rc) return rc;
-        chain(tail_post_kernel, n_sm * 2, 256, 0, s)(ovf, fin, L.n_vars, bm, L.vff, fvff, L.first_fault, fff, e0);
+        chain(tail_post_kernel, n_sm * 2, 256, 0, s)(gate, ovf + (cur ^ 1), fst, st, L.n_vars, bm, L.vff, fvff, L.first_fault, fff,
+                                                      e0);
         if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
-        cur ^= 1;
         e0 = e1;
     }
     if (L.profile & 2) profile_end(s);

@@ -170,9 +170,17 @@ int launch_bucket_check(const SortedCheck& C, cudaStream_t s);
 int launch_ss_radix(uint32_t* const key[2], uint32_t* const val[2], const int64_t* n_dev, int64_t cap,
                     int32_t n_vars, void* scratch, const int* gate, cudaStream_t s, int* passes);
 // Ops [0, n) of a trace as pairs for launch_sorted_check, checked for bad
-// bytes, ids out of range and GT without its EN; F written to step[0, n).
+// bytes, ids out of range and GT without its EN; F written to step[0, n); the
+// start state of the check as SortedStart says (n > 0).
+struct SortedStart {
+    int32_t* vff;               // [n_vars] := -1
+    int64_t* ff;                // := -1
+    uint8_t* status;            // [n_vars] := init, or (V,I)
+    const uint8_t* init;        // nullable
+    int* gate;                  // := 0
+};
 int launch_ss_keys(const uint8_t* kind_side, const int32_t* var, int64_t n, int64_t n_after, int32_t n_vars,
-                   uint32_t* key, uint32_t* val, uint8_t* step, int* err, cudaStream_t s);
+                   uint32_t* key, uint32_t* val, uint8_t* step, const SortedStart& z, int* err, cudaStream_t s);
 // enable >= 0: switch phase counting on/off and zero the counters; host_out
 // (nullable): copy the 8 counters (cycles summed over CTAs).
 int scan_phase_profile(int enable, unsigned long long* host_out);
