@@ -44,7 +44,7 @@ constexpr int64_t TF_LONG_CHUNKS_FROM = (int64_t)1 << 27;
 constexpr int TF_SLOT_DIV = 4;
 constexpr int64_t TF_HALF_TO = (int64_t)1 << 24;
 constexpr int64_t CAND_MAX = (int64_t)1 << 27;   // and at most 2^27 (set index << 4 fits 32 bits)
-constexpr int TF_PER = 16;                // ops per lane and step
+constexpr int TF_SUB = 4;                 // parts of 128 ops in a warp's step
 constexpr int TAIL_MIN_VARS = 16385;      // fewer variables take the reduce / carry / apply path
 constexpr int TAIL_MAX_VARS = 1 << 20;    // bitmap of 128 KB in shared memory
 constexpr int DEFAULT_FIRST_LOG2 = 21;    // first part 2^21 ops,
@@ -124,7 +124,7 @@ struct TailLayout {
     int64_t K = 0;        // pairs the sort buffers hold: the first part or an epoch's candidates
     size_t st0, st1, bm, cnt, off, coff, ncand, ovf, fvff, fff;
     size_t region;        // shared region: pairs and slots, or the fallback scan
-    size_t key0, val0, pos, key1, val1, sks, svar, spos, scratch;   // offsets inside the region
+    size_t key0, val0, pos, key1, val1, slot, scratch;   // offsets inside the region
     size_t total;
 };
 
@@ -170,11 +170,9 @@ TailLayout tail_layout(const TailShape& sh, int32_t n_vars, int64_t n_ops)
     const size_t shared_at = r;
     t.key1 = shared_at;
     t.val1 = shared_at + align_up(4 * K, 256);
+    t.slot = shared_at;
     const size_t second = 2 * align_up(4 * K, 256);
-    t.sks = shared_at;
-    t.svar = t.sks + align_up(n_slots, 256);
-    t.spos = t.svar + align_up(4 * n_slots, 256);
-    const size_t slots = align_up(n_slots, 256) + align_up(4 * n_slots, 256) + align_up(2 * n_slots, 256);
+    const size_t slots = align_up(8 * n_slots, 256);
     r += second > slots ? second : slots;
     size_t reg = r;
     const size_t fallback = scan_workspace_bytes(Emax, n_vars, false);
@@ -202,9 +200,7 @@ struct FilterParams {
     const uint32_t* bm;         // stuck bitmap at the epoch's start
     int bm_words;
     uint8_t* step;              // the epoch's outputs
-    uint8_t* sks;               // candidate slots, `slots` per chunk
-    int32_t* svar;
-    uint16_t* spos;             // position within the chunk
+    uint2* slot;                // candidate slots, `slots` per chunk
     uint32_t* cnt;              // candidates per chunk
     int* ovf;                   // set when a chunk has more candidates than slots
     int* err;
@@ -212,13 +208,31 @@ struct FilterParams {
     int slots;
 };
 
-// Each warp takes chunks of CHUNK ops in steps of 32 x 16 (lane L: ops
-// [16 L, 16 L + 16) of a step: one 16-byte load of op bytes and four of ids);
+// A GT must be followed by the EN of the same side on another variable (op i of
+// the epoch; other kinds pass).
+__device__ __forceinline__ void check_gt(const FilterParams& q, int64_t i)
+{
+    const uint32_t ks = q.kind_side[i];
+    if ((ks & 15u) != AMC_K_GT) return;
+    const int32_t v = (uint32_t)q.var[i] < (uint32_t)q.n_vars ? q.var[i] : 0;
+    const bool next = i + 1 < q.n_after;
+    const uint32_t nks = next ? q.kind_side[i + 1] : 0xFFu;
+    if (!((nks & 15) == AMC_K_EN && (nks >> 4) == (ks >> 4) && (next ? q.var[i + 1] : v) != v))
+        raise_error(q.err, AMC_E_INVALID);
+}
+
+// Each warp takes chunks of CHUNK ops in steps of 4 x 128 (lane L: ops 4 L to 4 L +
+// 3 of each 128, so that every load and store of the warp is one run of memory);
 // every position gets F (the candidates' statuses that are not F are written
-// after their check), the ops on variables outside the bitmap are staged in
-// the chunk's slots in position order.  Op bytes and ids are checked as in the
-// scan (malformed bytes, ids out of range, GT not followed by its EN); an id
-// out of range is staged as 0.
+// after their check), the ops on variables outside the bitmap are staged in the
+// chunk's slots in position order (id, position in the chunk << 8 | op byte).  Op
+// bytes and ids are checked as in the scan (malformed bytes, ids out of range, GT
+// not followed by its EN); an id out of range is staged as 0.
+// What bounds it: memory in the late epochs, where almost nothing is staged, the
+// L1 with its 32 bitmap look-ups in shared memory a warp load in the early ones.
+// Sixteen ops in a row per lane, staged as a byte, a word and two bytes: 1,197 us for
+// the five epochs of a 2^30-op trace (6.4 GB), 1,127 this way (6.0 TB/s in the two
+// long ones).
 template <int CHUNK>
 __global__ void __launch_bounds__(TF_THREADS, 1) tail_filter_kernel(const FilterParams q)
 {
@@ -229,138 +243,108 @@ __global__ void __launch_bounds__(TF_THREADS, 1) tail_filter_kernel(const Filter
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     const int64_t n_chunks = (q.n + CHUNK - 1) / CHUNK;
+    constexpr uint32_t F4 = 0x01010101u * ST_F;
     for (int64_t c = (int64_t)blockIdx.x * (TF_THREADS / 32) + warp; c < n_chunks;
          c += (int64_t)gridDim.x * (TF_THREADS / 32)) {
         const int64_t c0 = c * CHUNK;
         const int cn = (int)min((int64_t)CHUNK, q.n - c0);
         int wcount = 0;
         bool full = false;                                   // slots exhausted (warp-uniform)
-        for (int s0 = 0; s0 < cn; s0 += 32 * TF_PER) {
-            const int off = s0 + lane * TF_PER;              // offset in the chunk
-            const int64_t i0 = c0 + off;                     // offset in the epoch
-            const int nl = (int)min((int64_t)TF_PER, q.n - i0);
-            const bool vec = nl == TF_PER && q.bulk_ok;
-            uint32_t kw[TF_PER / 4];
-            int32_t va[TF_PER];
-            uint32_t liveMask = 0;
-            if (vec) {
-                // full step: four op bytes per 32-bit word are checked at once
-                const uint4 kk = __ldcs(reinterpret_cast<const uint4*>(q.kind_side + i0));
-                kw[0] = kk.x;
-                kw[1] = kk.y;
-                kw[2] = kk.z;
-                kw[3] = kk.w;
+        for (int s0 = 0; s0 < cn; s0 += 128 * TF_SUB) {
+            uint32_t kw[TF_SUB];
+            int4 va[TF_SUB];
+            uint32_t live = 0;                               // bit 4 t + j: op j of the lane's four in part t
+            if (q.bulk_ok && cn - s0 >= 128 * TF_SUB) {
+                const int64_t i0 = c0 + s0 + 4 * lane;       // offset in the epoch
 #pragma unroll
-                for (int h = 0; h < TF_PER / 4; ++h) {
-                    const int4 v4 = __ldcs(reinterpret_cast<const int4*>(q.var + i0) + h);
-                    va[4 * h] = v4.x;
-                    va[4 * h + 1] = v4.y;
-                    va[4 * h + 2] = v4.z;
-                    va[4 * h + 3] = v4.w;
+                for (int t = 0; t < TF_SUB; ++t) {
+                    kw[t] = __ldcs(reinterpret_cast<const uint32_t*>(q.kind_side + i0 + 128 * t));
+                    va[t] = __ldcs(reinterpret_cast<const int4*>(q.var + i0 + 128 * t));
                 }
-                uint32_t badk = 0, gt = 0, badv = 0;
+                // four op bytes per 32-bit word are checked at once
+                uint32_t badk = 0, gt = 0;
+                bool badv = false;
 #pragma unroll
-                for (int h = 0; h < TF_PER / 4; ++h) {
+                for (int t = 0; t < TF_SUB; ++t) {
                     // a valid byte has bits 3 and 5-7 clear (kinds 0..7, side bit 4)
-                    badk |= kw[h] & 0xE8E8E8E8u;
+                    badk |= kw[t] & 0xE8E8E8E8u;
                     // bytes whose kind is GT (6): zero bytes of (kind ^ 6)
-                    const uint32_t x = (kw[h] & 0x0F0F0F0Fu) ^ 0x06060606u;
+                    const uint32_t x = (kw[t] & 0x0F0F0F0Fu) ^ 0x06060606u;
                     gt |= (x - 0x01010101u) & ~x & 0x80808080u;
-                }
+                    int* const v4 = reinterpret_cast<int*>(&va[t]);
 #pragma unroll
-                for (int u = 0; u < TF_PER; ++u) {
-                    const uint32_t v = (uint32_t)va[u];
-                    const bool ok = v < (uint32_t)q.n_vars;
-                    badv |= !ok;
-                    const uint32_t uv = ok ? v : 0u;
-                    va[u] = (int32_t)uv;
-                    const uint32_t stuck = (sbm[uv >> 5] >> (uv & 31)) & 1u;
-                    liveMask |= (stuck ^ 1u) << u;
+                    for (int j = 0; j < 4; ++j) {
+                        const bool ok = (uint32_t)v4[j] < (uint32_t)q.n_vars;
+                        badv |= !ok;
+                        const uint32_t uv = ok ? (uint32_t)v4[j] : 0u;
+                        v4[j] = (int)uv;
+                        const uint32_t stuck = (sbm[uv >> 5] >> (uv & 31)) & 1u;
+                        live |= (stuck ^ 1u) << (4 * t + j);
+                    }
+                    __stcs(reinterpret_cast<uint32_t*>(q.step + i0 + 128 * t), F4);
                 }
                 if (badk) raise_error(q.err, AMC_E_INVALID);
                 if (badv) raise_error(q.err, AMC_E_RANGE);
-                if (gt) {
-                    // GT must be followed by EN of the same side on another variable
-#pragma unroll
-                    for (int u = 0; u < TF_PER; ++u) {
-                        const uint32_t ks = (kw[u >> 2] >> (8 * (u & 3))) & 0xFFu;
-                        if ((ks & 15u) != AMC_K_GT) continue;
-                        const uint32_t uv = (uint32_t)va[u] < (uint32_t)q.n_vars ? (uint32_t)va[u] : 0u;
-                        uint32_t nks = 0xFF;
-                        int32_t nv = (int32_t)uv;
-                        if (i0 + u + 1 < q.n_after) {
-                            nks = q.kind_side[i0 + u + 1];
-                            nv = q.var[i0 + u + 1];
-                        }
-                        if (!((nks & 15) == AMC_K_EN && (nks >> 4) == (ks >> 4) && nv != (int32_t)uv))
-                            raise_error(q.err, AMC_E_INVALID);
-                    }
-                }
-                constexpr uint32_t F4 = 0x01010101u * ST_F;
-                __stcs(reinterpret_cast<uint4*>(q.step + i0), make_uint4(F4, F4, F4, F4));
+                if (gt)
+                    for (int t = 0; t < TF_SUB; ++t)
+                        for (int j = 0; j < 4; ++j) check_gt(q, i0 + 128 * t + j);
             } else {
 #pragma unroll
-                for (int h = 0; h < TF_PER / 4; ++h) kw[h] = 0;
+                for (int t = 0; t < TF_SUB; ++t) {
+                    kw[t] = 0;
+                    va[t] = make_int4(0, 0, 0, 0);
+                    int* const v4 = reinterpret_cast<int*>(&va[t]);
 #pragma unroll
-                for (int u = 0; u < TF_PER; ++u) {
-                    va[u] = 0;
-                    if (u < nl) {
-                        kw[u >> 2] |= (uint32_t)q.kind_side[i0 + u] << (8 * (u & 3));
-                        va[u] = q.var[i0 + u];
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < TF_PER; ++u) {
-                    const uint32_t ks = (kw[u >> 2] >> (8 * (u & 3))) & 0xFFu;
-                    if (u < nl) {
+                    for (int j = 0; j < 4; ++j) {
+                        const int off = s0 + 128 * t + 4 * lane + j;
+                        if (off >= cn) continue;
+                        const int64_t i = c0 + off;
+                        const uint32_t ks = q.kind_side[i];
+                        kw[t] |= ks << (8 * j);
+                        v4[j] = q.var[i];
                         if ((ks & 0xE0u) || (ks & 15u) > AMC_K_EN) raise_error(q.err, AMC_E_INVALID);
-                        uint32_t uv = (uint32_t)va[u];
-                        if (va[u] < 0 || va[u] >= q.n_vars) {
+                        if (v4[j] < 0 || v4[j] >= q.n_vars) {
                             raise_error(q.err, AMC_E_RANGE);
-                            uv = 0;
+                            v4[j] = 0;
                         }
-                        if ((ks & 15u) == AMC_K_GT) {
-                            uint32_t nks = 0xFF;
-                            int32_t nv = (int32_t)uv;
-                            if (i0 + u + 1 < q.n_after) {
-                                nks = q.kind_side[i0 + u + 1];
-                                nv = q.var[i0 + u + 1];
-                            }
-                            if (!((nks & 15) == AMC_K_EN && (nks >> 4) == (ks >> 4) && nv != (int32_t)uv))
-                                raise_error(q.err, AMC_E_INVALID);
-                        }
-                        va[u] = (int32_t)uv;
-                        if (!((sbm[uv >> 5] >> (uv & 31)) & 1u)) liveMask |= 1u << u;
-                        q.step[i0 + u] = (uint8_t)ST_F;
+                        check_gt(q, i);
+                        const uint32_t uv = (uint32_t)v4[j];
+                        if (!((sbm[uv >> 5] >> (uv & 31)) & 1u)) live |= 1u << (4 * t + j);
+                        q.step[i] = (uint8_t)ST_F;
                     }
                 }
             }
-            const int cl = __popc(liveMask);
-            if (full || !__any_sync(0xffffffffu, cl != 0)) continue;
-            int pre = 0, wtot = 0;
+            if (full || !__any_sync(0xffffffffu, live != 0)) continue;
+            int at[TF_SUB], tot = 0;                         // the lane's first slot of each part
 #pragma unroll
-            for (int bit = 0; bit < 6; ++bit) {                 // counts 0..32
-                const uint32_t bal = __ballot_sync(0xffffffffu, (cl >> bit) & 1);
-                pre += __popc(bal & lt) << bit;
-                wtot += __popc(bal) << bit;
+            for (int t = 0; t < TF_SUB; ++t) {
+                const int cl = __popc((live >> (4 * t)) & 15u);
+                at[t] = tot;
+#pragma unroll
+                for (int bit = 0; bit < 3; ++bit) {          // counts 0..4
+                    const uint32_t bal = __ballot_sync(0xffffffffu, (cl >> bit) & 1);
+                    at[t] += __popc(bal & lt) << bit;
+                    tot += __popc(bal) << bit;
+                }
             }
-            if (wcount + wtot > q.slots) {
+            if (wcount + tot > q.slots) {
                 // more candidates than slots: the epoch is rechecked whole
                 if (lane == 0) atomicExch(q.ovf, 1);
                 full = true;
                 continue;
             }
-            int64_t idx = c * q.slots + wcount + pre;
+            uint2* const slot = q.slot + c * q.slots + wcount;
 #pragma unroll
-            for (int u = 0; u < TF_PER; ++u) {
-                if (liveMask & (1u << u)) {
-                    q.sks[idx] = (uint8_t)((kw[u >> 2] >> (8 * (u & 3))) & 0xFFu);
-                    q.svar[idx] = va[u];
-                    q.spos[idx] = (uint16_t)(off + u);
-                    ++idx;
-                }
+            for (int t = 0; t < TF_SUB; ++t) {
+                const int* const v4 = reinterpret_cast<const int*>(&va[t]);
+                int o = at[t];
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (live & (1u << (4 * t + j)))
+                        slot[o++] = make_uint2((uint32_t)v4[j], (uint32_t)(s0 + 128 * t + 4 * lane + j) << 8 |
+                                                                    ((kw[t] >> (8 * j)) & 0xFFu));
             }
-            wcount += wtot;
+            wcount += tot;
         }
         if (lane == 0) q.cnt[c] = (uint32_t)wcount;
     }
@@ -462,9 +446,7 @@ __global__ void __launch_bounds__(1024) tail_offsets_kernel(const uint32_t* __re
 // contiguous in the compacted set: lane L copies entries L, L + 32, ... of
 // that stretch (the stores coalesce), finding each entry's chunk by a binary
 // search over the G chunks' prefix counts, which lanes 0..G-1 hold.
-__global__ void __launch_bounds__(256) tail_gather_kernel(const uint8_t* __restrict__ sks,
-                                                          const int32_t* __restrict__ svar,
-                                                          const uint16_t* __restrict__ spos,
+__global__ void __launch_bounds__(256) tail_gather_kernel(const uint2* __restrict__ slot,
                                                           const uint32_t* __restrict__ cnt,
                                                           const uint32_t* __restrict__ coff, int n_chunks,
                                                           uint32_t* __restrict__ ckey, uint32_t* __restrict__ cval,
@@ -500,9 +482,10 @@ __global__ void __launch_bounds__(256) tail_gather_kernel(const uint8_t* __restr
                 const int64_t ch = g * G + k;
                 const int64_t src = ch * slots + (idx - first);
                 const uint32_t o = base + idx;
-                ckey[o] = (uint32_t)svar[src];
-                cval[o] = o << 4 | sorted_code_of(sks[src]);
-                cpos[o] = (uint32_t)ch * (uint32_t)chunk + spos[src];
+                const uint2 x = slot[src];
+                ckey[o] = x.x;
+                cval[o] = o << 4 | sorted_code_of(x.y & 0xFFu);
+                cpos[o] = (uint32_t)ch * (uint32_t)chunk + (x.y >> 8);
             }
         }
     }
@@ -596,9 +579,7 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
     int32_t* fvff = reinterpret_cast<int32_t*>(w + lay.fvff);
     int64_t* fff = reinterpret_cast<int64_t*>(w + lay.fff);
     uint8_t* reg = w + lay.region;
-    uint8_t* sks = reg + lay.sks;
-    int32_t* svar = reinterpret_cast<int32_t*>(reg + lay.svar);
-    uint16_t* spos = reinterpret_cast<uint16_t*>(reg + lay.spos);
+    uint2* slot = reinterpret_cast<uint2*>(reg + lay.slot);
     uint32_t* key0 = reinterpret_cast<uint32_t*>(reg + lay.key0);
     uint32_t* val0 = reinterpret_cast<uint32_t*>(reg + lay.val0);
     uint32_t* key1 = reinterpret_cast<uint32_t*>(reg + lay.key1);
@@ -666,15 +647,12 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
         q.bm = bm;
         q.bm_words = bm_words;
         q.step = L.step + e0;
-        q.sks = sks;
-        q.svar = svar;
-        q.spos = spos;
+        q.slot = slot;
         q.cnt = cnt;
         q.ovf = gate;
         q.slots = slots;
         q.err = L.err;
-        q.bulk_ok = ((uintptr_t)q.kind_side % 16 == 0) && ((uintptr_t)q.var % 16 == 0) &&
-                    ((uintptr_t)q.step % 16 == 0);
+        q.bulk_ok = (uintptr_t)q.kind_side % 4 == 0 && (uintptr_t)q.var % 16 == 0 && (uintptr_t)q.step % 4 == 0;
         const int n_chunks = (int)chunks_of(n);
         const int fgrid = (int)min((int64_t)n_sm, ((int64_t)n_chunks + TF_THREADS / 32 - 1) / (TF_THREADS / 32));
         if (chunk == TF_CHUNK)
@@ -689,7 +667,7 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
         while (G < 32 && n_chunks / (2 * G) >= 8192) G *= 2;
         const int64_t groups = ((int64_t)n_chunks + G - 1) / G;
         const int ggrid = (int)min((int64_t)n_sm * 8, (groups + 7) / 8);
-        chain(tail_gather_kernel, ggrid, 256, 0, s)(sks, svar, spos, cnt, coff, n_chunks, key0, val0, cpos, G, chunk, slots,
+        chain(tail_gather_kernel, ggrid, 256, 0, s)(slot, cnt, coff, n_chunks, key0, val0, cpos, G, chunk, slots,
                                                  gate);
         if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
         // the candidates, at most C (count on the device), from the epoch's

@@ -1,7 +1,8 @@
 """GPU parity of the epoch path around the candidate slots: chunks of 1,024 ops
 with exactly as many ops on variables that are not stuck as there are slots (half
 of a chunk in epochs of at most 2^24 ops, a quarter in longer ones), one fewer,
-and one more, which rechecks the epoch whole.  Bit-exact against the oracle."""
+and one more, which rechecks the epoch whole; arrays that start off the filter's
+vector alignment.  Bit-exact against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -38,6 +39,31 @@ def test_slots(amc, oracle_mod, monkeypatch, epoch, per_chunk):
     var[live] = STUCK + rng.integers(0, ALIVE, int(live.sum()))
     exp = oracle_mod.check_trace(ks, var, STUCK + ALIVE, None)
     out = amc.check_trace(torch.from_numpy(ks).cuda(), torch.from_numpy(var).cuda(), STUCK + ALIVE)
+    assert amc.sync_status() == 0
+    assert np.array_equal(out["step_status"].cpu().numpy(), exp[0])
+    assert np.array_equal(out["final_status"].cpu().numpy(), exp[1])
+    assert np.array_equal(out["var_first_fault"].cpu().numpy(), exp[2])
+    assert int(out["first_fault"].cpu()[0]) == exp[3]
+
+
+@pytest.mark.parametrize("shift", [(0, 0, 0), (1, 0, 0), (0, 1, 0), (0, 0, 1), (4, 4, 4), (3, 2, 1)])
+def test_alignment(amc, oracle_mod, monkeypatch, shift):
+    """kind_side, var and step_status so many elements off a 256-byte boundary."""
+    monkeypatch.setenv("AMC_SCAN_TAIL", "13,-1")
+    rng = np.random.default_rng(5)
+    n, nv = 100_003, 20_000
+    ks = rng.choice(np.array([0, 1, 2, 3, 4, 5, 16, 17, 18, 19, 20, 21], np.uint8), n)
+    var = (nv * rng.random(n) ** 3).astype(np.int32)
+    exp = oracle_mod.check_trace(ks, var, nv, None)
+    d_ks = torch.zeros(n + 8, dtype=torch.uint8, device="cuda")[shift[0]:shift[0] + n]
+    d_var = torch.zeros(n + 8, dtype=torch.int32, device="cuda")[shift[1]:shift[1] + n]
+    d_ks.copy_(torch.from_numpy(ks))
+    d_var.copy_(torch.from_numpy(var))
+    out = dict(step_status=torch.empty(n + 8, dtype=torch.uint8, device="cuda")[shift[2]:shift[2] + n],
+               final_status=torch.empty(nv, dtype=torch.uint8, device="cuda"),
+               var_first_fault=torch.empty(nv, dtype=torch.int32, device="cuda"),
+               first_fault=torch.empty(1, dtype=torch.int64, device="cuda"))
+    amc.check_trace(d_ks, d_var, nv, out=out)
     assert amc.sync_status() == 0
     assert np.array_equal(out["step_status"].cpu().numpy(), exp[0])
     assert np.array_equal(out["final_status"].cpu().numpy(), exp[1])
