@@ -25,7 +25,7 @@ constexpr int MAX_ELEMS = 32;
 // byte maps to an element id; comp[a][b] is "a then b"; app[a][s] applies a
 // to status s.  Built on the host (monoid.cu) from the effect rules and passed
 // to kernels by value.
-struct Tables {
+struct alignas(16) Tables {
     uint8_t comp[MAX_ELEMS * MAX_ELEMS];
     uint8_t app[MAX_ELEMS * 8];
     uint8_t elem_of[256];           // op byte -> element id / ELEM_BAD / ELEM_GT

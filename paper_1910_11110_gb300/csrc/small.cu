@@ -4,15 +4,22 @@
 // For traces of at most SMALL_MAX_OPS ops over at most SMALL_MAX_VARS
 // variables, one launch of one CTA does the whole check: its 32 warps take
 // consecutive stretches of the trace; (1) each warp folds its stretch into
-// one transfer function per variable (32 ops at a time, lanes with the same
-// variable grouped by match.any, the group's first lane composing them in
-// order), kept in shared memory; (2) a thread per variable carries the
-// initial status through the warps' functions, giving every stretch its entry
-// statuses and the final status; (3) each warp re-runs its stretch from those
+// one transfer function per variable (32 ops at a time: the lanes with the same
+// variable are found by a ballot per bit of the id, and compose their functions
+// in log steps), kept in shared memory; (2) the initial status is carried through
+// the warps' functions (a warp per variable, its lanes composing in log steps, for
+// few variables, else a thread per variable), giving every stretch its entry
+// statuses and the final status; (3) each warp takes its stretch from those
 // statuses and writes every op's status and the first faults.  No workspace,
 // no memset, one kernel: the latency of a check is one launch.  The initial
 // and final statuses may share a buffer: a variable's initial status is read
 // and its final status written by the same thread in step (2).
+// What bounds it is latency: four batches are loaded at once, and a stretch of at
+// most four stays in registers between (1) and (3).  4,096 ops over 16 variables:
+// 10.1 us with a load per batch, match.any and a serial chain over equal lanes,
+// 6.3 us this way.
+#include <cstddef>
+
 #include "amc_internal.cuh"
 #include "scan_trace.cuh"
 
@@ -23,12 +30,17 @@ namespace {
 constexpr int SMALL_MAX_OPS = 1 << 16;
 constexpr int SMALL_MAX_VARS = 2048;
 constexpr int SNW = 32;                      // warps
+constexpr int SB = 4;                        // batches of 32 ops loaded at once
+// Up to so many variables a warp carries one in five steps of about 60 cycles, a
+// warp's share of them one after another; above, 1,024 threads one each in 32.
+constexpr int SMALL_SCAN_VARS = 128;
+
+static_assert(SNW == 32, "the carry's lanes are the stretches");
 
 struct SmallSmem {
     uint8_t comp[MAX_ELEMS * MAX_ELEMS];
     uint8_t app[MAX_ELEMS * 8];
     uint8_t elem_of[256];
-    uint8_t mb[SNW][32];
     uint8_t row[SNW][SMALL_MAX_VARS];        // per warp: folded functions, then current statuses
     unsigned long long ff;
 };
@@ -44,83 +56,136 @@ __global__ void __launch_bounds__(SNW * 32, 1) small_trace_kernel(const uint8_t*
     SmallSmem& S = *reinterpret_cast<SmallSmem*>(smraw);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const uint32_t lt = lanemask_lt();
-    for (int i = tid; i < MAX_ELEMS * MAX_ELEMS; i += SNW * 32) S.comp[i] = tab.comp[i];
-    for (int i = tid; i < MAX_ELEMS * 8; i += SNW * 32) S.app[i] = tab.app[i];
-    for (int i = tid; i < 256; i += SNW * 32) S.elem_of[i] = tab.elem_of[i];
+    // the tables, a word at a time (lanes reading different parameter words take turns)
+    static_assert(offsetof(Tables, app) % 4 == 0 && offsetof(Tables, elem_of) % 4 == 0 && sizeof(Tables) % 4 == 0, "");
+    for (int i = tid; i < MAX_ELEMS * MAX_ELEMS / 4; i += SNW * 32)
+        reinterpret_cast<uint32_t*>(S.comp)[i] = reinterpret_cast<const uint32_t*>(tab.comp)[i];
+    for (int i = tid; i < MAX_ELEMS * 8 / 4; i += SNW * 32)
+        reinterpret_cast<uint32_t*>(S.app)[i] = reinterpret_cast<const uint32_t*>(tab.app)[i];
+    for (int i = tid; i < 256 / 4; i += SNW * 32)
+        reinterpret_cast<uint32_t*>(S.elem_of)[i] = reinterpret_cast<const uint32_t*>(tab.elem_of)[i];
     const uint32_t ID = tab.identity;
     for (int v = lane; v < n_vars; v += 32) S.row[w][v] = (uint8_t)ID;
     if (tid == 0) S.ff = ~0ull;
-    __syncthreads();
     const int per = (n + SNW - 1) / SNW;
     const int lo = min(n, w * per), hi = min(n, lo + per);
-    // (1) fold each stretch per variable
-    for (int b = lo; b < hi; b += 32) {
-        const int i = b + lane;
-        const bool ok = i < hi;
-        const uint32_t ks = ok ? kind_side[i] : 0u;
-        int32_t v = ok ? var[i] : 0;
+    const int bits = 32 - __clz(n_vars - 1 | 1);
+    // SB batches of 32 ops: byte and id; then the op's function after those of the
+    // lanes before it with its variable (inc), and theirs alone (exc)
+    uint32_t ks[SB], inc[SB], exc[SB];
+    int32_t var_of[SB];
+    bool last[SB];                                       // no later lane of the batch has the variable
+    auto load = [&](int b) {
+#pragma unroll
+        for (int u = 0; u < SB; ++u) {
+            const int i = b + 32 * u + lane;
+            ks[u] = i < hi ? kind_side[i] : 0u;
+            var_of[u] = i < hi ? var[i] : 0;
+        }
+    };
+    auto functions = [&](int b, int u, bool check) {
+        const bool ok = b + 32 * u + lane < hi;
+        int32_t v = var_of[u];
         uint32_t m = ID;
         if (ok) {
             if (v < 0 || v >= n_vars) {
-                raise_error(err, AMC_E_RANGE);
+                if (check) raise_error(err, AMC_E_RANGE);
                 v = 0;
             }
-            m = S.elem_of[ks];
+            m = S.elem_of[ks[u]];
             if (m == ELEM_BAD || m == ELEM_GT) {         // GT only in a guarded check
-                raise_error(err, AMC_E_INVALID);
+                if (check) raise_error(err, AMC_E_INVALID);
                 m = ID;
             }
         }
-        S.mb[w][lane] = (uint8_t)m;
-        const uint32_t peers = __match_any_sync(0xffffffffu, ok ? (uint32_t)v : 0xFFFFFFFFu);
-        __syncwarp();
-        if (ok && lane == __ffs(peers) - 1) {
-            uint32_t acc = S.row[w][v];
-            for (uint32_t q = peers; q; q &= q - 1) acc = S.comp[acc * MAX_ELEMS + S.mb[w][__ffs(q) - 1]];
-            S.row[w][v] = (uint8_t)acc;
+        var_of[u] = v;
+        uint32_t peers = __ballot_sync(0xffffffffu, ok);
+        for (int k = 0; k < bits; ++k) {
+            const uint32_t x = __ballot_sync(0xffffffffu, (v >> k) & 1);
+            peers &= (v >> k) & 1 ? x : ~x;
         }
-        __syncwarp();
+        if (!ok) peers = 1u << lane;
+        const int before = (peers & lt) ? 31 - __clz(peers & lt) : -1;
+        uint32_t f = m;
+        for (int q = before; __any_sync(0xffffffffu, q >= 0);) {
+            const uint32_t fq = __shfl_sync(0xffffffffu, f, q & 31);
+            const int qq = __shfl_sync(0xffffffffu, q, q & 31);
+            if (q >= 0) {
+                f = S.comp[fq * MAX_ELEMS + f];
+                q = qq;
+            }
+        }
+        const uint32_t e = __shfl_sync(0xffffffffu, f, before & 31);
+        inc[u] = f;
+        exc[u] = before >= 0 ? e : ID;
+        last[u] = ok && !(peers & ~lt & ~(1u << lane));
+    };
+    load(lo);
+    __syncthreads();
+    // (1) fold each stretch per variable
+    for (int b = lo; b < hi; b += 32 * SB) {
+        if (b > lo) load(b);
+#pragma unroll
+        for (int u = 0; u < SB; ++u) {
+            if (b + 32 * u >= hi) break;
+            functions(b, u, true);
+            if (last[u]) S.row[w][var_of[u]] = S.comp[S.row[w][var_of[u]] * MAX_ELEMS + inc[u]];
+            __syncwarp();
+        }
     }
     __syncthreads();
     // (2) carry: entry status of every stretch, final statuses
-    for (int v = tid; v < n_vars; v += SNW * 32) {
-        uint32_t s = init ? (uint32_t)(init[v] & 7u) : (uint32_t)AMC_ST_VI;
-        for (int k = 0; k < SNW; ++k) {
-            const uint32_t e = S.row[k][v];
-            S.row[k][v] = (uint8_t)s;
-            s = S.app[e * 8 + s];
+    if (n_vars <= SMALL_SCAN_VARS) {
+        for (int v = w; v < n_vars; v += SNW) {
+            const uint32_t s0 = init ? (uint32_t)(init[v] & 7u) : (uint32_t)AMC_ST_VI;
+            uint32_t f = S.row[lane][v];
+#pragma unroll
+            for (int d = 1; d < SNW; d <<= 1) {
+                const uint32_t x = __shfl_up_sync(0xffffffffu, f, d);
+                if (lane >= d) f = S.comp[x * MAX_ELEMS + f];
+            }
+            const uint32_t out = S.app[f * 8 + s0], in = __shfl_up_sync(0xffffffffu, out, 1);
+            S.row[lane][v] = (uint8_t)(lane ? in : s0);
+            if (lane == SNW - 1) {
+                fin[v] = (uint8_t)out;
+                vff[v] = -1;
+            }
         }
-        fin[v] = (uint8_t)s;
-        vff[v] = -1;
+    } else {
+        for (int v = tid; v < n_vars; v += SNW * 32) {
+            uint32_t s = init ? (uint32_t)(init[v] & 7u) : (uint32_t)AMC_ST_VI;
+            for (int k = 0; k < SNW; ++k) {
+                const uint32_t e = S.row[k][v];
+                S.row[k][v] = (uint8_t)s;
+                s = S.app[e * 8 + s];
+            }
+            fin[v] = (uint8_t)s;
+            vff[v] = -1;
+        }
     }
     __syncthreads();
     // (3) statuses of every op from the stretch's entry statuses
-    for (int b = lo; b < hi; b += 32) {
-        const int i = b + lane;
-        const bool ok = i < hi;
-        const uint32_t ks = ok ? kind_side[i] : 0u;
-        int32_t v = ok ? var[i] : 0;
-        if (v < 0 || v >= n_vars) v = 0;
-        uint32_t m = ok ? S.elem_of[ks] : ID;
-        if (m == ELEM_BAD || m == ELEM_GT) m = ID;
-        S.mb[w][lane] = (uint8_t)m;
-        const uint32_t peers = __match_any_sync(0xffffffffu, ok ? (uint32_t)v : 0xFFFFFFFFu);
-        __syncwarp();
-        const uint32_t cur = ok ? S.row[w][v] : 0u;
-        __syncwarp();
-        if (ok) {
-            uint32_t acc = ID;
-            for (uint32_t q = peers & lt; q; q &= q - 1) acc = S.comp[acc * MAX_ELEMS + S.mb[w][__ffs(q) - 1]];
-            const uint32_t pre = S.app[acc * 8 + cur];
-            const uint32_t post = S.app[S.comp[acc * MAX_ELEMS + m] * 8 + cur];
-            step[i] = (uint8_t)post;
-            if (post == ST_F && pre != ST_F) {
-                vff[v] = i;                              // a variable becomes stuck once
-                atomicMin(&S.ff, (unsigned long long)i);
+    for (int b = lo; b < hi; b += 32 * SB) {
+        if (hi - lo > 32 * SB) load(b);
+#pragma unroll
+        for (int u = 0; u < SB; ++u) {
+            if (b + 32 * u >= hi) break;
+            if (hi - lo > 32 * SB) functions(b, u, false);
+            const int i = b + 32 * u + lane;
+            const int32_t v = var_of[u];
+            const uint32_t cur = i < hi ? S.row[w][v] : 0u;
+            const uint32_t pre = S.app[exc[u] * 8 + cur], post = S.app[inc[u] * 8 + cur];
+            __syncwarp();
+            if (last[u]) S.row[w][v] = (uint8_t)post;
+            if (i < hi) {
+                step[i] = (uint8_t)post;
+                if (post == ST_F && pre != ST_F) {
+                    vff[v] = i;                          // a variable becomes stuck once
+                    atomicMin(&S.ff, (unsigned long long)i);
+                }
             }
-            if (lane == 31 - __clz(peers)) S.row[w][v] = (uint8_t)post;
+            __syncwarp();
         }
-        __syncwarp();
     }
     __syncthreads();
     if (tid == 0) *first_fault = S.ff == ~0ull ? -1 : (int64_t)S.ff;
