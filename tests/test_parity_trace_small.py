@@ -20,7 +20,7 @@ def amc():
 @pytest.mark.parametrize("n", [1, 31, 32, 33, 1024, 1025, 4095, 4096, 4097, 8192, 65_535, 65_536])
 @pytest.mark.parametrize("n_vars", [1, 2, 3, 16, 17, 127, 128, 129, 2047, 2048])
 def test_small(amc, oracle_mod, monkeypatch, n, n_vars):
-    monkeypatch.setenv("AMC_AUTOTUNE", "0")
+    monkeypatch.setenv("AMC_TRACE_CANDIDATE", "0")               # the path by size
     rng = np.random.default_rng(n * 4096 + n_vars)
     ks = rng.choice(np.array([0, 1, 2, 3, 4, 5, 16, 17, 18, 19, 20, 21], np.uint8), n,
                     p=[.02, .3, .05, .05, .1, .05, .02, .16, .05, .05, .1, .05])
