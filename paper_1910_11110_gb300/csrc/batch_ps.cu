@@ -641,9 +641,9 @@ __device__ void run_part(const PsParams& p, int64_t prog, uint32_t (*rows)[2][32
     int32_t pl = 0, npl = 0;
     uint32_t runs = 0;                                     // ops on other variables than g
     uint32_t own = 0;                                      // the lane's own among them
-    uint32_t rotx = 0, stuck = 0;                          // the token's op
+    uint32_t wrong = 0;                                    // variable out of range
+    uint32_t word = 0;                                     // the token's op: rotx | statuses that get stuck << 20
     int to = -1;                                           // place after the part it announces (-1: none in the program)
-    bool valid = false;
     while (pos < len && !bad) {
         if (pos >= wb + 32 || pos < wb) {
             if (pos == wb + 32) {
@@ -661,7 +661,8 @@ __device__ void run_part(const PsParams& p, int64_t prog, uint32_t (*rows)[2][32
             const bool op = ps_is_op(ks), opx = op && !(pl == g && g >= 0);
             runs = __ballot_sync(0xffffffffu, opx);
             if (!op && w == 0 && lane < len - wb) step[wb + lane] = 0;
-            valid = pl >= 0 && pl < nv;
+            const bool valid = pl >= 0 && pl < nv;
+            wrong = __ballot_sync(0xffffffffu, opx && !valid);
             own = __ballot_sync(0xffffffffu, opx && valid && (pl >> 5) == w);
 #pragma unroll
             for (int b = 0; b < 5; ++b) {
@@ -669,36 +670,40 @@ __device__ void run_part(const PsParams& p, int64_t prog, uint32_t (*rows)[2][32
                 own &= (lane >> b) & 1 ? m : ~m;
             }
             const uint32_t o = op ? ((ks & 15u) << 1) | (ks >> 4) : 0u;
-            rotx = T.rotx[o];
-            stuck = T.stuck[o];
+            word = T.rotx[o] | (T.stuck[o] & 15u) << 20;
             to = pl >= 0 && pl < len - wb - lane - 1 ? wb + lane + 1 + pl : -1;
         }
+        // the run of ops from here on (at most to the window's end), and the token
+        // after it
         const int off = pos - wb;
         const uint32_t left = runs >> off;
-        if (left & 1u) {
-            // the run of ops from here on (at most to the window's end)
-            const int cnt = ~left ? __ffs(~left) - 1 : 32;
+        const int cnt = ~left ? __ffs(~left) - 1 : 32;
+        const uint32_t k0 = __shfl_sync(0xffffffffu, ks, off + cnt);
+        const int next = __shfl_sync(0xffffffffu, to, off + cnt);
+        if (cnt) {
             const uint32_t run = (cnt < 32 ? (1u << cnt) - 1u : ~0u) << off;
-            if (((run >> lane) & 1u) && !valid) {
+            if (run & wrong) {
                 range = true;
-                if (w == 0) step[wb + lane] = 0;
+                if (w == 0 && ((run & wrong) >> lane & 1u)) step[wb + lane] = 0;
             }
+            // a lane's ops in order, the next one's word fetched while one is applied
             uint32_t mine = own & run;
-            for (int n = __reduce_max_sync(0xffffffffu, __popc(mine)); n > 0; --n) {
-                const int L = __ffs(mine) - 1;             // (-1: any word will do)
-                const uint32_t x = __shfl_sync(0xffffffffu, rotx, L), st = __shfl_sync(0xffffffffu, stuck, L);
+            uint32_t x = __shfl_sync(0xffffffffu, word, __ffs(mine) - 1);       // (none: any word will do)
+            while (__any_sync(0xffffffffu, mine != 0)) {
+                const uint32_t rest = mine & (mine - 1);
+                const uint32_t xn = __shfl_sync(0xffffffffu, word, __ffs(rest) - 1);
                 if (mine) {
-                    if (J & st) ff = min(ff, wb + L);
+                    const int at = wb + __ffs(mine) - 1;
+                    if (J & ((x >> 20) * 0x108421u)) ff = min(ff, at);
                     J = op_on_x(J, x);
-                    step[wb + L] = (uint8_t)proj(J);
-                    mine &= mine - 1;
+                    step[at] = (uint8_t)proj(J);
                 }
+                mine = rest;
+                x = xn;
             }
             pos += cnt;
-            continue;
+            if (off + cnt >= 32 || pos >= len) continue;
         }
-        const uint32_t k0 = __shfl_sync(0xffffffffu, ks, off);
-        const int next = __shfl_sync(0xffffffffu, to, off);
         const uint32_t c = (f.meta >> 4) & 3u;
         uint32_t(*const row)[32] = rows[max(depth - 1, 0)];
         if (k0 == AMC_T_END) {
