@@ -1034,7 +1034,7 @@ def measure_kloc(args, amc, dev):
     return {"workload": "kloc_trace", "k": k, "n_ops": n, "n_vars": nv, "seed": 6, "ms_per_step": ms,
             "ops_per_s": n / (ms * 1e-3),
             "roofline": roofline(alg, ms, note="algorithmic bytes: 5 B per op in, 1 B per op out, 5 B per variable"),
-            "gpu_launches_per_step": 11,
+            "gpu_launches_per_step": kloc_launches(n, nv),
             "cpu_baseline": {"value": reps * m / dt, "unit": UNIT, "cores": 1, "kind": "oracle",
                              "sample": f"the first {m} ops, {reps} pass(es), single thread ({dt:.1f} s)"},
             "clocks": clk}
@@ -1213,6 +1213,24 @@ def guarded_check_launches(n_statements, n_vars):
     if path in ("warp_dense", "dense"):
         return 5 if n_vars <= 65_536 else 2 * n
     return 1 + 2
+
+
+def kloc_launches(n_ops, n_vars):
+    """Kernels of one k-location check: pairs, the sort (three kernels per radix
+    pass) and the scan.  In epochs (at most 2^20 variables, 2^22 ops or more, a
+    quarter of them beyond the first part): the stuck bitmap, and per epoch, each
+    ending at four times its start, the filter, a three-kernel scan, the
+    compaction, sort and scan."""
+    sort = 3 * radix_passes(n_vars) + 1
+    first = 1 << 17
+    while first < min(2 * n_vars, 1 << 21):
+        first *= 2
+    if n_ops < 1 << 22 or n_vars > 1 << 20 or 4 * first > n_ops:
+        return 1 + sort
+    epochs = 0
+    while first < n_ops:
+        first, epochs = 4 * first, epochs + 1
+    return 1 + sort + 1 + epochs * (1 + 3 + 1 + sort)
 
 
 def vectorpu_launches(n_statements, n_vars):
