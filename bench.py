@@ -1191,15 +1191,17 @@ def radix_passes(key_range):
     return (kb + 6) // 7
 
 
-def overlap_launches(n_arrays, lifetimes=False):
-    """Kernels that build the overlap lists.  Without lifetimes, up to 8,192
-    arrays: counts, a three-kernel scan, the total, the lists and the overflow
-    clear.  Else: keys, the sort by range start (three kernels per radix pass),
-    the counting sweep, a three-kernel scan, the total, the cursor reset, the
-    filling sweep, two sorts of the pairs, the copy and the overflow clear."""
-    if not lifetimes and n_arrays <= 8192:
+def overlap_launches(n_arrays, n_lists=None):
+    """Kernels that build the overlap lists.  Without lifetimes (n_lists None), up
+    to 8,192 arrays: counts, a three-kernel scan, the total, the lists and the
+    overflow clear.  Else: keys, the counts' reset, the sort by range start (three
+    kernels per radix pass), the counting sweep, a three-kernel scan, the total,
+    the cursor reset, the filling sweep, the sorts of the pairs by other and by
+    list, the copy and the overflow clear."""
+    if n_lists is None and n_arrays <= 8192:
         return 7
-    return 1 + 3 * radix_passes(2 ** 31 - 1) + 1 + 3 + 1 + 1 + 1 + 2 * 3 * radix_passes(n_arrays) + 1 + 1
+    sorts = radix_passes(2 ** 31 - 1) + radix_passes(n_arrays) + radix_passes(n_lists or n_arrays)
+    return 1 + 1 + 1 + 3 + 1 + 1 + 1 + 3 * sorts + 1 + 1
 
 
 def guarded_check_launches(n_statements, n_vars):
@@ -1245,7 +1247,7 @@ def lifetimes_launches(n_arrays, n_calls, n_statements):
     emission and the total; then two guarded checks with the inheritance
     kernel between them."""
     births = 1 + 3 * radix_passes(n_calls + 1)
-    return (overlap_launches(n_arrays, lifetimes=True) + births + 1 + 3 + 1 + 1 +
+    return (overlap_launches(n_arrays, n_arrays * min(n_calls, 256)) + births + 1 + 3 + 1 + 1 +
             2 * guarded_check_launches(n_statements, 2 * n_arrays) + 1)
 
 
