@@ -566,9 +566,12 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
     if (!tail_shape(L.n_ops, L.n_vars, false, sh, L.tail)) return AMC_E_INVALID;
     const TailLayout lay = tail_layout(sh, L.n_vars, L.n_ops);
     uint8_t* w = static_cast<uint8_t*>(L.workspace);
-    // the statuses as the trace goes on, where they are wanted in the end; a
-    // fallback's final ones
-    uint8_t* st = L.final_status ? L.final_status : w + lay.st0;
+    // the statuses as the trace goes on, where they are wanted in the end unless
+    // the initial ones lie there too (the first part reads those while it writes
+    // its final ones); a fallback's final ones
+    const bool apart = L.final_status && !(L.init && L.init < L.final_status + L.n_vars &&
+                                           L.final_status < L.init + L.n_vars);
+    uint8_t* st = apart ? L.final_status : w + lay.st0;
     uint8_t* fst = w + lay.st1;
     uint32_t* bm = reinterpret_cast<uint32_t*>(w + lay.bm);
     uint32_t* cnt = reinterpret_cast<uint32_t*>(w + lay.cnt);
@@ -718,6 +721,9 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
         if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
         e0 = e1;
     }
+    if (L.final_status && !apart &&
+        cudaMemcpyAsync(L.final_status, st, (size_t)L.n_vars, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+        return AMC_E_CUDA;
     if (L.profile & 2) profile_end(s);
     return AMC_OK;
 }

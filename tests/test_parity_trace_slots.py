@@ -69,3 +69,28 @@ def test_alignment(amc, oracle_mod, monkeypatch, shift):
     assert np.array_equal(out["final_status"].cpu().numpy(), exp[1])
     assert np.array_equal(out["var_first_fault"].cpu().numpy(), exp[2])
     assert int(out["first_fault"].cpu()[0]) == exp[3]
+
+
+@pytest.mark.parametrize("mix", [[0.002, 0.6, 0.1, 0.1, 0.198], [0.2, 0.4, 0.15, 0.15, 0.1]])
+def test_statuses_in_place(amc, oracle_mod, monkeypatch, mix):
+    """Requests of a session whose statuses are read and written in one buffer:
+    variables with runs over several sort tiles of the first part."""
+    import test_serve
+    import workloads
+
+    monkeypatch.setenv("AMC_SCAN_TAIL", "16,-1")
+    rng = np.random.default_rng(17)
+    nv = 20_000
+    reqs = []
+    for n in (200_003, 70_001, 150_000):
+        ks, var = workloads.trace_random(rng, n, nv, p=mix)
+        var[rng.random(n) < 0.3] = 11                  # a run of a third of the ops
+        reqs.append((0, ks, var))
+    sessions = [(0, nv, reqs)]
+    exp, fin = test_serve.oracle_results(oracle_mod, sessions)
+    got, got_fin = test_serve.run_server(amc, sessions, 2, True)
+    for k, (step, ff, _) in exp.items():
+        assert got[k]["error"] == 0
+        assert np.array_equal(got[k]["status"], step), k
+        assert got[k]["first_fault"] == ff, k
+    assert np.array_equal(got_fin[0], fin[0])
