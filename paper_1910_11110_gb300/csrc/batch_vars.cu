@@ -152,6 +152,9 @@ __device__ void run_program(const BatchParams& p, int64_t prog, VarSmem& S, uint
                 const uint32_t says = to | (ks == AMC_T_IF ? AN_ELSE : 0u) | (ks == AMC_T_WHILE ? AN_WHILE : 0u);
                 const int level = opn ? depth : els ? depth - 1 : -1;       // of the construct it speaks for
                 bool wrong = in && !op && !opn && !els && !enb;
+                // more constructs than a balanced program of its length can have, and
+                // than its share of C holds (the words behind it are the next program's)
+                wrong |= nc + __popc(O) > len / 2;
                 wrong |= (opn || els) && (to == NIL16 || level < 0 || level >= AMC_MAX_DEPTH);
                 const int most = min(__reduce_max_sync(0xffffffffu, in ? depth + opn : 0), AMC_MAX_DEPTH);
                 uint32_t heard = NIL16;                    // in force at the token's own construct
@@ -296,7 +299,7 @@ __device__ void run_program(const BatchParams& p, int64_t prog, VarSmem& S, uint
                 uint32_t c = opened[q];
                 uint64_t cw;
                 do cw = construct(--c);
-                while ((int)c_depth(cw) != depth);
+                while (c && (int)c_depth(cw) != depth);
                 if (depth) below[depth - 1] = f;
                 ++depth;
                 f.end = c_end(cw);
