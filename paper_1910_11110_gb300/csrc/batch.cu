@@ -315,10 +315,12 @@ struct Plan {
     uint8_t* rsave;               // [reduce warps][2][AMC_MAX_DEPTH][seg_max] reduce-pass copies
     int64_t* ord_off;             // [P + 1] apply units before the k-th program of the queue order
     int simple;                   // no program can be split: one unit per program, no planning
-    const int* gate;              // nullable: set when a program is left to these kernels (else they do nothing)
+    const int* gate;              // nullable: [0] set when a program is left to these kernels (else they do
+                                  // nothing), [1] when all are (malformed token offsets)
 };
 
-__device__ __forceinline__ bool gated_off(const int* gate) { return gate && *gate == 0; }
+__device__ __forceinline__ bool gated_off(const int* gate) { return gate && gate[0] == 0; }
+__device__ __forceinline__ bool all_left(const int* gate) { return gate && gate[1] != 0; }
 
 __device__ __forceinline__ int64_t split_slots(int64_t len, int32_t nv, int64_t split)
 {
@@ -439,7 +441,7 @@ __global__ void __launch_bounds__(BWARPS * 32, MINB) batch_kernel(const BatchPar
             if (lane == 0) raise_error(p.err, AMC_E_INVALID);
             continue;
         }
-        if (pl.gate && program_fits_vars(pt1 - pt0, nv, p.split)) continue;     // evaluated variable by variable
+        if (pl.gate && !all_left(pl.gate) && program_fits_vars(pt1 - pt0, nv, p.split)) continue;   // evaluated variable by variable
         if (nv <= SMEM_VARS)
             run_unit<true>(p, u, S, tab);
         else
@@ -458,6 +460,7 @@ __global__ void __launch_bounds__(1024) plan_offsets_kernel(const int64_t* __res
                                                             const int* gate)
 {
     if (gated_off(gate)) return;
+    if (all_left(gate)) split = INT64_MAX;                 // no program is cut: its extents may be anything
     __shared__ unsigned long long tmp_s[32], tmp_u[32];
     __shared__ unsigned long long carry_s, carry_u;
     if (threadIdx.x == 0) {
@@ -595,21 +598,25 @@ __device__ __forceinline__ int cost_bucket(int64_t len, int32_t nv)
     return 62 - min(max(k, 0), 62);
 }
 
-// With `others`, also notes whether a program is not evaluated variable by
-// variable.
+// With `gate`, also notes whether a program is not evaluated variable by
+// variable, and whether one has malformed token offsets: its neighbours may then
+// have tokens in common, and so the scratch rows that evaluation by variables
+// keeps positions in; a set read from another program's row is only a wrong set.
 __global__ void bucket_count_kernel(const int64_t* __restrict__ tok_off, const int32_t* __restrict__ nvars, int64_t n,
-                                    int32_t* __restrict__ counts, int64_t split, int* others)
+                                    int64_t n_tokens, int32_t* __restrict__ counts, int64_t split, int* gate)
 {
     __shared__ int32_t c[64];
     if (threadIdx.x < 64) c[threadIdx.x] = 0;
     __syncthreads();
-    bool other = false;
+    bool other = false, bad = false;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t len = tok_off[i + 1] - tok_off[i];
-        atomicAdd(&c[cost_bucket(len, nvars[i])], 1);
-        other |= !program_fits_vars(len, nvars[i], split);
+        const int64_t a = tok_off[i], b = tok_off[i + 1];
+        atomicAdd(&c[cost_bucket(b - a, nvars[i])], 1);
+        other |= !program_fits_vars(b - a, nvars[i], split);
+        bad |= a < 0 || b < a || b > n_tokens;
     }
-    if (others && other) *others = 1;
+    if (gate && (other || bad)) gate[0] = 1;
+    if (gate && bad) gate[1] = 1;
     __syncthreads();
     if (threadIdx.x < 64 && c[threadIdx.x]) atomicAdd(&counts[threadIdx.x], c[threadIdx.x]);
 }
@@ -811,14 +818,14 @@ int launch_batch(const BatchLaunch& B, cudaStream_t s)
     // and nothing when there is none
     const bool by_vars = p.save_rows == AMC_MAX_DEPTH;
     unsigned long long* vars_queue = reinterpret_cast<unsigned long long*>(p.queue_head) + 1;
-    int* others = reinterpret_cast<int*>(p.queue_head + 2);
-    pl.gate = by_vars ? others : nullptr;
+    int* gate = reinterpret_cast<int*>(p.queue_head + 2);
+    pl.gate = by_vars ? gate : nullptr;
     if (B.profile & 1) profile_begin(s);
     if (cudaMemsetAsync(p.queue_head, 0, 24, s) != cudaSuccess) return AMC_E_CUDA;
     if (cudaMemsetAsync(counts, 0, 256, s) != cudaSuccess) return AMC_E_CUDA;
     if (B.longest_first || by_vars)
-        bucket_count_kernel<<<128, 256, 0, s>>>(B.prog_tok_off, B.prog_nvars, B.n_progs, counts, p.split,
-                                                by_vars ? others : nullptr);
+        bucket_count_kernel<<<128, 256, 0, s>>>(B.prog_tok_off, B.prog_nvars, B.n_progs, B.n_tokens, counts, p.split,
+                                                by_vars ? gate : nullptr);
     if (!pl.simple) {
         plan_offsets_kernel<<<1, 1024, 0, s>>>(B.prog_tok_off, B.prog_nvars, B.n_progs,
                                                const_cast<int64_t*>(pl.slot_off), const_cast<int64_t*>(pl.unit_off),
@@ -836,7 +843,7 @@ int launch_batch(const BatchLaunch& B, cudaStream_t s)
         p.order = order;
     }
     if (by_vars) {
-        const int rc = launch_batch_vars(p, B.max_ctas, vars_queue, s);
+        const int rc = launch_batch_vars(p, B.max_ctas, vars_queue, gate + 1, s);
         if (rc) return rc;
     }
     if (!pl.simple) {

@@ -71,8 +71,8 @@ __device__ __forceinline__ bool program_by_vars(const BatchParams& p, int64_t pr
     return program_fits_vars(b - a, nv, p.split);
 }
 // Those programs of the batch (p.save / p.alt with AMC_MAX_DEPTH rows: 8 bytes
-// a token each); *queue is zero.
-int launch_batch_vars(const BatchParams& p, int64_t max_ctas, unsigned long long* queue, cudaStream_t s);
+// a token each); *queue is zero.  None when *off (device) is set.
+int launch_batch_vars(const BatchParams& p, int64_t max_ctas, unsigned long long* queue, const int* off, cudaStream_t s);
 
 size_t batch_workspace_bytes(int64_t n_tokens, int64_t n_progs);
 size_t batch_workspace_bytes(int64_t n_tokens, int64_t n_progs, bool no_split, int save_rows);

@@ -350,8 +350,9 @@ __device__ void run_program(const BatchParams& p, int64_t prog, VarSmem& S, uint
 }
 
 __global__ void __launch_bounds__(VWARPS * 32, VCTAS) vars_kernel(const __grid_constant__ BatchParams p,
-                                                             unsigned long long* queue)
+                                                             unsigned long long* queue, const int* off)
 {
+    if (*off) return;
     extern __shared__ __align__(16) uint8_t smem[];
     VarSmem& S = *reinterpret_cast<VarSmem*>(smem);
     for (int i = threadIdx.x; i < 16 * 32; i += blockDim.x) S.img[i] = p.tab.img[i];
@@ -372,7 +373,7 @@ __global__ void __launch_bounds__(VWARPS * 32, VCTAS) vars_kernel(const __grid_c
 
 }  // namespace
 
-int launch_batch_vars(const BatchParams& p, int64_t max_ctas, unsigned long long* queue, cudaStream_t s)
+int launch_batch_vars(const BatchParams& p, int64_t max_ctas, unsigned long long* queue, const int* off, cudaStream_t s)
 {
     int dev = 0, n_sm = 0;
     cudaGetDevice(&dev);
@@ -383,7 +384,7 @@ int launch_batch_vars(const BatchParams& p, int64_t max_ctas, unsigned long long
     const int64_t need = (p.n_progs + VWARPS - 1) / VWARPS;
     if (grid > need) grid = need;
     if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
-    vars_kernel<<<(unsigned)grid, VWARPS * 32, sizeof(VarSmem), s>>>(p, queue);
+    vars_kernel<<<(unsigned)grid, VWARPS * 32, sizeof(VarSmem), s>>>(p, queue, off);
     return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
 }
 

@@ -64,3 +64,25 @@ def test_open_constructs(amc, oracle_mod, opener, n_open, n_ops):
         progs += [(tok, pay, 1), p] + ([(tok[:0], pay[:0], 1)] if i % 3 else [(tok[-1:], pay[-1:], 1)])
         good += [False, True, True]
     check_among(amc, oracle_mod, progs, good)
+
+
+@pytest.mark.parametrize("n_tokens_more", [0, 70_000])
+def test_common_tokens(amc, oracle_mod, n_tokens_more):
+    # offsets that go back, so that two programs have tokens in common, offsets
+    # before the first and behind the last token: refused, and the programs that
+    # share nothing as the oracle has them
+    good = programs(40, seed=95)
+    tok, pay = np.concatenate([p[0] for p in good]), np.concatenate([p[1] for p in good])
+    a = offsets([p[0].size for p in good])
+    n = int(a[-1])
+    more = np.full(200 + n_tokens_more, NOOP, np.uint8)
+    tok, pay = np.concatenate([tok, more]), np.concatenate([pay, np.zeros(more.size, np.int32)])
+    back = [n + 100, n + 50, n + 150, -5, n + 150, 1 << 40, n, tok.size]
+    off = np.concatenate([a, np.array(back, np.int64)])
+    nv = np.array([p[2] for p in good] + [1] * len(back), np.int32)
+    out, rc = run(amc, tok, pay, off, nv)
+    assert rc == amc.E_INVALID
+    step, final, pff = oracle_mod.check_batch(tok[:n], pay[:n], a, nv[:40])
+    assert np.array_equal(out["step_mask"][:n], step)
+    assert np.array_equal(out["final_mask"][:int(nv[:40].sum())], final)
+    assert np.array_equal(out["prog_first_fault"][:40], pff)
