@@ -269,7 +269,9 @@ __device__ __forceinline__ int64_t translate_call(const TrParams& p, Sink out, i
         }
     }
     if (p.infer && declared == 1 && !EMIT && !LIFE) {
-        // counting a single list: its entries but the call's arguments
+        // counting a single list: its entries but the call's arguments, which are
+        // looked up as emission meets them (of malformed arrays a pair may overlap
+        // and not be listed)
 #pragma unroll U
         for (int i = 0; i < NMAX; ++i) {
             if (i >= n) break;
@@ -278,7 +280,13 @@ __device__ __forceinline__ int64_t translate_call(const TrParams& p, Sink out, i
 #pragma unroll U
             for (int j = 0; j < NMAX; ++j) {
                 if (j >= n) break;
-                args += j != i && st[i] < en[j] && st[j] < en[i];
+                int32_t a = 0, b = len[i];
+                while (a < b) {
+                    const int32_t m = (a + b) >> 1;
+                    if ((int32_t)(q[i][m] >> 1) < arr[j]) a = m + 1;
+                    else b = m;
+                }
+                args += a < len[i] && (int32_t)(q[i][a] >> 1) == arr[j];
             }
             o += 3 * (len[i] - args);
         }
@@ -458,7 +466,8 @@ __global__ void __launch_bounds__(TNT, EMIT ? 6 : 10) calls_kernel(const TrParam
     for (int i = 0; i < TOPND; ++i) {
         arr[i] = -1;
         mode[i] = 0;
-        st[i] = en[i] = len[i] = 0;
+        st[i] = en[i] = INT32_MAX;                      // no operand: meets no range
+        len[i] = 0;
         lo[i] = 0;
         if (i < n) {
             arr[i] = p.opnd_array[k0 + i];
