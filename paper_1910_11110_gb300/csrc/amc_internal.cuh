@@ -3,9 +3,10 @@
 #pragma once
 
 #include <cuda_runtime.h>
-
-#include <utility>
 #include <stdint.h>
+
+#include <atomic>
+#include <utility>
 
 #include "amc.h"
 
@@ -221,6 +222,23 @@ __device__ __forceinline__ uint32_t lanes_with_same(uint32_t v, bool ok, bool lo
         rest &= ~m;
     }
     return peers;
+}
+
+// Lets KERNEL take up to `most` bytes of dynamic shared memory: the most that any
+// launch of it asks for.  The limit is the kernel's, one per device, so that a
+// call that set its own smaller size could lower it between another thread's
+// setting and its launch.  False when that fails.
+template <auto KERNEL>
+bool allow_smem(size_t most)
+{
+    static std::atomic<uint64_t> done{0};                 // a bit per device
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const uint64_t bit = dev < 64 ? (uint64_t)1 << dev : 0;
+    if (done.load(std::memory_order_relaxed) & bit) return true;
+    if (cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) return false;
+    done.fetch_or(bit, std::memory_order_relaxed);
+    return true;
 }
 
 // Kernels of one call follow each other on its stream: chain(kernel, grid, block,

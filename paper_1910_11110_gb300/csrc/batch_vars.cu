@@ -378,8 +378,7 @@ int launch_batch_vars(const BatchParams& p, int64_t max_ctas, unsigned long long
     int dev = 0, n_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaFuncSetAttribute(vars_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(VarSmem)) != cudaSuccess)
-        return AMC_E_CUDA;
+    if (!allow_smem<vars_kernel>(sizeof(VarSmem))) return AMC_E_CUDA;
     int64_t grid = VCTAS * (int64_t)n_sm;
     const int64_t need = (p.n_progs + VWARPS - 1) / VWARPS;
     if (grid > need) grid = need;

@@ -497,8 +497,7 @@ int launch_kloc(const KlocLaunch& L, cudaStream_t s)
     }
     if (S) {
         const size_t smem = 4 * (size_t)((L.n_vars + 31) / 32);
-        if (cudaFuncSetAttribute(kl_filter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return AMC_E_CUDA;
+        if (!allow_smem<kl_filter_kernel>(KEPOCH_MAX_VARS / 8)) return AMC_E_CUDA;
         chain(kl_bitmap_kernel, (unsigned)((L.n_vars + 255) / 256), 256, 0, s)(L.final_status, L.n_vars, bm);
         int32_t* cnt = reinterpret_cast<int32_t*>(w + lay.cnt);
         int64_t* off = reinterpret_cast<int64_t*>(w + lay.off);

@@ -39,7 +39,6 @@ constexpr int DNW = DNT / 32;
 constexpr int DPOS = 12;                 // log2(DT): position bits of a key
 constexpr int DDIG = 7;                  // radix digit bits
 constexpr int DENSE_MAX_VARS = 16384;    // by size up to here
-constexpr int WARP_MAX_VARS = 8192;      // three-kernel carry up to here
 constexpr int64_t DENSE_MIN_OPS = 1 << 10;
 
 __device__ __forceinline__ int dpad(int i) { return i + (i >> 5); }
@@ -479,9 +478,7 @@ int launch_dense_range(const ScanLaunch& L, int max_chunks, int64_t n_follow, ui
     const size_t smem = sizeof(DenseSmem);
     auto kr = dense_chunk_kernel<false>;
     auto ka = dense_chunk_kernel<true>;
-    if (cudaFuncSetAttribute(kr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return AMC_E_CUDA;
+    if (!allow_smem<dense_chunk_kernel<false>>(smem) || !allow_smem<dense_chunk_kernel<true>>(smem)) return AMC_E_CUDA;
     if (L.profile & 1) profile_begin(s);
     kr<<<p.n_chunks, DNT, smem, s>>>(p);
     if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
@@ -651,7 +648,7 @@ namespace {
 bool owner_wide(int32_t n_vars)
 {
     const char* e = getenv("AMC_SCAN_DENSE_SORT");
-    return n_vars > WARP_MAX_VARS || (e && e[0] == '1');
+    return n_vars > OWN_NARROW_VARS || (e && e[0] == '1');
 }
 
 }  // namespace

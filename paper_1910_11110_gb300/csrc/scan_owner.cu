@@ -628,12 +628,6 @@ int run_carry(OwnParams p, const OwnShape& S, bool one_carry, bool last, cudaStr
     return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
 }
 
-template <typename K>
-bool allow_smem(K* kernel, size_t bytes)
-{
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
-}
-
 template <int NO, int NS, int OPT>
 int run_owner(const ScanLaunch& L, const OwnShape& S, bool guarded, bool one_carry, uint8_t* ws, cudaStream_t s)
 {
@@ -642,8 +636,11 @@ int run_owner(const ScanLaunch& L, const OwnShape& S, bool guarded, bool one_car
     const size_t smS = sizeof(SortSmem<NO, NS, OPT>) + (size_t)S.row;
     const size_t smW = sizeof(WalkSmem<NO, TILE>) + (size_t)S.row;
     auto sort = guarded ? own_sort_kernel<NO, NS, OPT, true> : own_sort_kernel<NO, NS, OPT, false>;
-    if (!allow_smem(sort, smS) || !allow_smem(own_apply_kernel<NO, TILE>, smW) ||
-        (guarded && !allow_smem(own_resolve_kernel<NO, TILE>, smW)))
+    const size_t row = NO == 128 ? OWN_NARROW_VARS : OWN_MAX_VARS;       // the longest
+    const size_t mS = sizeof(SortSmem<NO, NS, OPT>) + row, mW = sizeof(WalkSmem<NO, TILE>) + row;
+    if (smS > mS || !allow_smem<own_sort_kernel<NO, NS, OPT, true>>(mS) ||
+        !allow_smem<own_sort_kernel<NO, NS, OPT, false>>(mS) || !allow_smem<own_apply_kernel<NO, TILE>>(mW) ||
+        !allow_smem<own_resolve_kernel<NO, TILE>>(mW))
         return AMC_E_CUDA;
     if (L.profile & 1) profile_begin(s);
     sort<<<(unsigned)S.n_chunks, NS, smS, s>>>(p);

@@ -8,6 +8,8 @@ namespace amc {
 
 // Variables whose statuses fit a CTA's shared memory beside a tile.
 constexpr int32_t OWN_MAX_VARS = 1 << 16;
+// ... with 128 owners.
+constexpr int32_t OWN_NARROW_VARS = 8192;
 
 // Scratch after the single-pass workspace (chunk rows); the sorted tiles take
 // the single-pass workspace itself.

@@ -879,15 +879,7 @@ int launch_bucket_check(const SortedCheck& C, cudaStream_t s)
     if (C.cap > ((int64_t)1 << 28) || !C.pos || !bucket_check_ok(C.n_vars)) return AMC_E_INVALID;
     const int W = bucket_width(C.n_vars);
     const size_t smem = (size_t)(BKW + 1) * W;
-    static size_t attr_set[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 64 || attr_set[dev] < smem) {
-        if (cudaFuncSetAttribute(ss_bucket_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess)
-            return AMC_E_CUDA;
-        if (dev < 64) attr_set[dev] = smem;
-    }
+    if (!allow_smem<ss_bucket_kernel>((size_t)(BKW + 1) * BK_MAX_W)) return AMC_E_CUDA;
     const int n_sm = sm_count();
     const int64_t tiles = (C.cap + ST - 1) / ST;
     auto grid = [&](int per_sm) { return (int)(tiles < (int64_t)n_sm * per_sm ? tiles : (int64_t)n_sm * per_sm); };

@@ -597,15 +597,9 @@ int launch_scan_tail(const ScanLaunch& L, cudaStream_t s)
     const int bm_words = (L.n_vars + 31) / 32;
     const size_t fsmem = 4 * (size_t)bm_words;
     if ((int)fsmem > max_optin) return AMC_E_INVALID;
-    static size_t attr_set[64] = {};
-    if (dev >= 64 || attr_set[dev] < fsmem) {
-        if (cudaFuncSetAttribute(tail_filter_kernel<TF_CHUNK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)fsmem) != cudaSuccess ||
-            cudaFuncSetAttribute(tail_filter_kernel<TF_CHUNK_SHORT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)fsmem) != cudaSuccess)
-            return AMC_E_CUDA;
-        if (dev < 64) attr_set[dev] = fsmem;
-    }
+    if (!allow_smem<tail_filter_kernel<TF_CHUNK>>(TAIL_MAX_VARS / 8) ||
+        !allow_smem<tail_filter_kernel<TF_CHUNK_SHORT>>(TAIL_MAX_VARS / 8))
+        return AMC_E_CUDA;
     if (L.profile & 1) profile_begin(s);
 
     // first part: ops [0, S) checked by sorting them by variable, from the

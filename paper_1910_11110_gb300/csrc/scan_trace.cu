@@ -1677,11 +1677,11 @@ int launch_kernel(ScanParams p, const ScanLaunch& L, cudaStream_t s)
     const int64_t room = ((int64_t)max_optin - (int64_t)sizeof(ScanSmem<KeyT, TILE, THREADS>) - 1024) / 16 * 4;
     if (p.fbw > room) p.fbw = room > 0 ? (int)room : 0;          // shared bitmap words (multiple of 4)
     const size_t smem = sizeof(ScanSmem<KeyT, TILE, THREADS>) + 4 * (size_t)p.fbw;
-    static size_t attr_set[64] = {};
-    if (dev >= 64 || attr_set[dev] != smem) {
-        if (cudaFuncSetAttribute(scan_trace_kernel<KeyT, TILE, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem) != cudaSuccess)
-            return AMC_E_CUDA;
+    if (!allow_smem<scan_trace_kernel<KeyT, TILE, THREADS>>(sizeof(ScanSmem<KeyT, TILE, THREADS>) +
+                                                            4 * (size_t)(room > 0 ? room : 0)))
+        return AMC_E_CUDA;
+    static std::atomic<size_t> carved[64] = {};               // size the carve-out was last asked for
+    if (dev >= 64 || carved[dev].load(std::memory_order_relaxed) != smem) {
         // ask for the smallest shared-memory carve-out that still holds the
         // resident CTAs, so that the rest of the SM's memory serves as L1 for
         // the stuck bitmap
@@ -1693,7 +1693,7 @@ int launch_kernel(ScanParams p, const ScanLaunch& L, cudaStream_t s)
             cudaFuncSetAttribute(scan_trace_kernel<KeyT, TILE, THREADS>,
                                  cudaFuncAttributePreferredSharedMemoryCarveout, pct);
         }
-        if (dev < 64) attr_set[dev] = smem;
+        if (dev < 64) carved[dev].store(smem, std::memory_order_relaxed);
     }
     int n_sm = 0, per_sm = 0;
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);

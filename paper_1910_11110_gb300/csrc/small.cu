@@ -201,15 +201,7 @@ bool scan_small_eligible(const ScanLaunch& L)
 
 int launch_scan_small(const ScanLaunch& L, cudaStream_t s)
 {
-    static bool attr_done[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 64 || !attr_done[dev]) {
-        if (cudaFuncSetAttribute(small_trace_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(SmallSmem)) != cudaSuccess)
-            return AMC_E_CUDA;
-        if (dev < 64) attr_done[dev] = true;
-    }
+    if (!allow_smem<small_trace_kernel>(sizeof(SmallSmem))) return AMC_E_CUDA;
     if (L.profile & 1) profile_begin(s);
     small_trace_kernel<<<1, SNW * 32, sizeof(SmallSmem), s>>>(L.kind_side, L.var, (int32_t)L.n_ops, L.n_vars, L.init,
                                                               L.step, L.final_status, L.vff, L.first_fault, L.err,
