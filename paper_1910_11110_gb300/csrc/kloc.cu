@@ -23,15 +23,20 @@
 // first (F is absorbing: on a long trace nearly every op sees it), and the
 // scan writes only the statuses that are not F.
 //
-// A trace of 2^22 ops or more over at most 2^20 variables is not sorted whole.
-// Its first part is (twice as many ops as variables, rounded up to a power of
-// two, 2^17 to 2^21); after that each epoch ends at four times its start, and
+// A trace of 2^23 ops or more over at most 2^20 variables is not sorted whole.
+// Its first 2^21 ops are; after that each epoch ends at four times its start, and
 // a streaming kernel writes F at every position of it and keeps, in position
 // order, the ops on variables that are not stuck (a bit per variable, in shared
 // memory); only those are sorted and scanned, from the statuses at the epoch's
 // start.  What bounded the whole sort is its three passes over 8 bytes an op:
 // 100,000,007 ops over 2^20 variables at k = 4, of which 94 % see F, took 3.92
-// ms that way and take 0.73 ms in epochs.
+// ms that way and take 0.64 ms in epochs.
+// Where nothing gets stuck epochs save nothing and each costs some dozen short
+// kernels: an epoch of which a sample of 4,096 ops has at least 7/8 on variables
+// that are not stuck is kept whole, without a compaction, and shorter traces are
+// sorted at once.  The same trace of writes alone: 4.45 ms sorted whole, 5.30 with
+// every epoch compacted, 4.43 so; 5,000,003 ops over 100 variables: 0.196
+// sorted whole, 0.371 in epochs from 2^17 ops on, 0.173 so.
 #include "amc_internal.cuh"
 #include "dscan.cuh"
 #include "kloc.cuh"
@@ -55,7 +60,8 @@ constexpr int KOP_SHIFT = 21;            // op byte in key bits 21-28 when n_var
 constexpr int KFT = 1024;                // filter threads (one CTA per SM: the bitmap fills shared memory)
 constexpr int KFE = 16;                  // ops per filter lane and stretch
 constexpr int KSTRETCH = 32 * KFE;
-constexpr int64_t KEPOCH_MIN_OPS = (int64_t)1 << 22;
+constexpr int64_t KFIRST = (int64_t)1 << 21;       // ops of the first part
+constexpr int64_t KEPOCH_MIN_OPS = 4 * KFIRST;
 constexpr int32_t KEPOCH_MAX_VARS = 1 << 20;
 
 __device__ __forceinline__ uint32_t kcomp(uint32_t f, uint32_t g)
@@ -158,9 +164,15 @@ struct KFilterParams {
     const uint32_t* bm;         // stuck at the epoch's start
     uint32_t* key;              // slots: the kept ops of stretch i from KSTRETCH i on, in position order
     uint32_t* val;
+    uint32_t* all_key;          // the ops of an epoch kept whole, at their positions in it
+    uint32_t* all_val;
     int32_t* cnt;               // kept ops per stretch
+    int* all;                   // out: the epoch is kept whole
+    const uint8_t* fin;         // statuses so far
+    uint8_t* st;                // out: a copy (the scan reads it while it writes the later ones)
     int* err;
 };
+constexpr int KSAMPLE = 4 * KFT;
 
 // A warp per stretch of 512 ops, 16 consecutive ops per lane, no barrier: 1,024
 // threads an SM stream beside the 128 KB bitmap.
@@ -173,6 +185,16 @@ __global__ void __launch_bounds__(KFT, 1) kl_filter_kernel(const __grid_constant
     for (int i = t; i < (p.n_vars + 31) / 32; i += KFT) sbm[i] = p.bm[i];
     if (t < 8) valid[t] = p.valid[t];
     __syncthreads();
+    // ops on variables that are not stuck, of a sample that is the same in every CTA
+    int alive = 0;
+#pragma unroll
+    for (int j = 0; j < KSAMPLE / KFT; ++j) {
+        const uint32_t v = (uint32_t)p.var[(int64_t)(j * KFT + t) * p.n / KSAMPLE];
+        alive += __syncthreads_count(v < (uint32_t)p.n_vars && !((sbm[v >> 5] >> (v & 31)) & 1u));
+    }
+    const bool all = 8 * alive >= 7 * KSAMPLE;
+    if (blockIdx.x == 0 && t == 0) *p.all = all;
+    for (int v = (int)blockIdx.x * KFT + t; v < p.n_vars; v += (int)gridDim.x * KFT) p.st[v] = p.fin[v];
     const int64_t ns = (p.n + KSTRETCH - 1) / KSTRETCH, nw = (int64_t)gridDim.x * (KFT / 32);
     const bool wide = (uintptr_t)p.op % 16 == 0 && (uintptr_t)p.var % 16 == 0 && (uintptr_t)p.step % 16 == 0;
     for (int64_t s = (int64_t)blockIdx.x * (KFT / 32) + (t >> 5); s < ns; s += nw) {
@@ -224,6 +246,27 @@ __global__ void __launch_bounds__(KFT, 1) kl_filter_kernel(const __grid_constant
         }
         if (bado) raise_error(p.err, AMC_E_INVALID);
         if (badv) raise_error(p.err, AMC_E_RANGE);
+        if (all) {
+            if (lane == 0) p.cnt[s] = (int32_t)min((int64_t)KSTRETCH, p.n - s * KSTRETCH);
+#pragma unroll
+            for (int h = 0; h < KFE / 4; ++h) {
+                uint32_t kk[4], vv[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    kk[u] = p.pack ? (v[4 * h + u] | ((o[h] >> (8 * u)) & 0xFFu) << KOP_SHIFT) : v[4 * h + u];
+                    vv[u] = (uint32_t)(p.offset + i0 + 4 * h + u);
+                    if (m < KFE && 4 * h + u < m) {
+                        p.all_key[i0 + 4 * h + u] = kk[u];
+                        p.all_val[i0 + 4 * h + u] = vv[u];
+                    }
+                }
+                if (m == KFE) {
+                    reinterpret_cast<uint4*>(p.all_key + i0)[h] = make_uint4(kk[0], kk[1], kk[2], kk[3]);
+                    reinterpret_cast<uint4*>(p.all_val + i0)[h] = make_uint4(vv[0], vv[1], vv[2], vv[3]);
+                }
+            }
+            continue;
+        }
         const int c = __popc(live), incl = warp_incl_sum(c);
         if (lane == 31) p.cnt[s] = incl;
         int64_t at = s * KSTRETCH + (incl - c);
@@ -238,13 +281,17 @@ __global__ void __launch_bounds__(KFT, 1) kl_filter_kernel(const __grid_constant
     }
 }
 
-// The kept ops of every stretch from its slots to their place; the total.
+// The kept ops of every stretch from its slots to their place (an epoch kept
+// whole is there already); the scan's tile words zeroed.
 __global__ void __launch_bounds__(256) kl_compact_kernel(const uint32_t* __restrict__ skey, const uint32_t* __restrict__ sval,
                                                          const int32_t* __restrict__ cnt, const int64_t* __restrict__ off,
                                                          int64_t ns, uint32_t* __restrict__ key,
-                                                         uint32_t* __restrict__ val)
+                                                         uint32_t* __restrict__ val, const int* all,
+                                                         uint32_t* __restrict__ zero, int n_zero)
 {
     follow();
+    for (int i = (int)(blockIdx.x * blockDim.x + threadIdx.x); i < n_zero; i += (int)(gridDim.x * blockDim.x)) zero[i] = 0;
+    if (*all) return;
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < ns; s += nw) {
@@ -403,14 +450,11 @@ __global__ void __launch_bounds__(KNT) kl_seg_kernel(const KSegParams p)
 // First part of a trace checked in epochs (0: the whole trace at once).
 int64_t first_part(int64_t n_ops, int32_t n_vars)
 {
-    if (n_ops < KEPOCH_MIN_OPS || n_vars > KEPOCH_MAX_VARS) return 0;
-    int64_t S = (int64_t)1 << 17;
-    while (S < 2 * (int64_t)n_vars && S < ((int64_t)1 << 21)) S <<= 1;
-    return 4 * S <= n_ops ? S : 0;
+    return n_ops < KEPOCH_MIN_OPS || n_vars > KEPOCH_MAX_VARS ? 0 : KFIRST;
 }
 
 struct KLayout {
-    size_t key0, val0, key1, val1, scratch, tstat, ctr, cnt, off, scan, st, bm, total;
+    size_t key0, val0, key1, val1, scratch, tstat, ctr, all, cnt, off, scan, st, bm, total;
 };
 
 KLayout klayout(int64_t n, int32_t n_vars)
@@ -427,6 +471,7 @@ KLayout klayout(int64_t n, int32_t n_vars)
     const bool epochs = first_part(n, n_vars) > 0;
     L.tstat = take(4 * (size_t)((n + KT - 1) / KT + 1));       // with ctr: zeroed before every scan
     L.ctr = take(4);
+    L.all = take(4);
     const int64_t ns = epochs ? (n + KSTRETCH - 1) / KSTRETCH : 0;
     L.cnt = take(4 * (size_t)ns);
     L.off = take(8 * ((size_t)ns + 1));
@@ -469,7 +514,7 @@ int launch_kloc(const KlocLaunch& L, cudaStream_t s)
         const int rc = launch_ss_radix(key, val, n_dev, n, L.n_vars, w + lay.scratch, nullptr, s, &passes);
         if (rc) return rc;
         const int64_t tiles = (n + KT - 1) / KT;
-        if (cudaMemsetAsync(w + lay.tstat, 0, lay.ctr + 4 - lay.tstat, s) != cudaSuccess) return AMC_E_CUDA;
+        if (!n_dev && cudaMemsetAsync(w + lay.tstat, 0, lay.ctr + 4 - lay.tstat, s) != cudaSuccess) return AMC_E_CUDA;
         KSegParams p;
         p.vmask = pack ? (1u << KOP_SHIFT) - 1u : 0xFFFFFFFFu;
         p.pack = pack;
@@ -516,11 +561,13 @@ int launch_kloc(const KlocLaunch& L, cudaStream_t s)
             q.bm = bm;
             q.key = key[1];
             q.val = val[1];
+            q.all_key = key[0];
+            q.all_val = val[0];
+            q.all = reinterpret_cast<int*>(w + lay.all);
             q.cnt = cnt;
             q.err = L.err;
-            // the scan reads the statuses at the epoch's start while it writes the later ones
-            if (cudaMemcpyAsync(w + lay.st, L.final_status, (size_t)L.n_vars, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-                return AMC_E_CUDA;
+            q.fin = L.final_status;
+            q.st = w + lay.st;
             const int64_t ns = (q.n + KSTRETCH - 1) / KSTRETCH;
             const int64_t fb = (ns + KFT / 32 - 1) / (KFT / 32), cb = (ns + 7) / 8;
             chain(kl_filter_kernel, (unsigned)(fb < n_sm ? fb : n_sm), KFT, smem, s)(q);
@@ -528,7 +575,9 @@ int launch_kloc(const KlocLaunch& L, cudaStream_t s)
             int rc = dscan_exclusive(cnt, off, ns, w + lay.scan, s);
             if (rc) return rc;
             chain(kl_compact_kernel, (unsigned)(cb < 8 * n_sm ? cb : 8 * n_sm), 256, 0, s)(key[1], val[1], cnt, off, ns, key[0],
-                                                                                     val[0]);
+                                                                                     val[0], q.all,
+                                                                                     reinterpret_cast<uint32_t*>(w + lay.tstat),
+                                                                                     (int)((lay.ctr + 4 - lay.tstat) / 4));
             if (cudaGetLastError() != cudaSuccess) return AMC_E_CUDA;
             rc = check(q.n, off + ns, w + lay.st);
             if (rc) return rc;
