@@ -252,6 +252,7 @@ bool allow_smem(size_t most)
 // 2^30 ops (74) 2076 -> 1955, four locations 708 -> 652.  The owner-sorted
 // tiles and the VectorPU translation are launched without it: a few kernels of
 // thousands of CTAs, where waiting CTAs only take room (5 M calls 4.02 -> 4.26 ms).
+// Not `ahead`: the same launch without it (sorts of many pairs).
 __device__ __forceinline__ void follow()
 {
     cudaTriggerProgrammaticLaunchCompletion();
@@ -262,6 +263,7 @@ template <typename... P>
 struct Chained {
     void (*kernel)(P...);
     cudaLaunchConfig_t config;
+    bool ahead;
     template <typename... A>
     void operator()(A&&... args)
     {
@@ -269,20 +271,20 @@ struct Chained {
         at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at.val.programmaticStreamSerializationAllowed = 1;
         config.attrs = &at;
-        config.numAttrs = 1;
+        config.numAttrs = ahead ? 1 : 0;
         cudaLaunchKernelEx(&config, kernel, std::forward<A>(args)...);
     }
 };
 
 template <typename... P>
-Chained<P...> chain(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s)
+Chained<P...> chain(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool ahead = true)
 {
     cudaLaunchConfig_t c = {};
     c.gridDim = grid;
     c.blockDim = block;
     c.dynamicSmemBytes = smem;
     c.stream = s;
-    return {kernel, c};
+    return {kernel, c, ahead};
 }
 
 }  // namespace amc
