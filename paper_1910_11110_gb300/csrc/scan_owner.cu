@@ -8,7 +8,9 @@
 // the owner: one ballot per bit ranks a warp's 32 ops), and then every thread
 // walks its own ops in order: a byte of shared memory per variable that no
 // other thread touches, so there is no grouping of lanes with equal variables,
-// no composition within a group and no barrier inside the walk.
+// no composition within a group and no barrier inside the walk.  Where one owner
+// has much of a tile (a trace that is mostly about a few variables) a warp walks
+// its ops in up to 32 pieces instead, with a row of the owner's bytes per piece.
 //   1. sort + reduce: CTA c takes chunk c (consecutive tiles): every tile is
 //      checked, sorted by owner and written out as 4-byte entries (variable,
 //      4-bit op code, position); each thread folds its ops into one transfer
@@ -45,7 +47,16 @@ namespace {
 
 constexpr int POSB = 12;                  // position bits of an entry
 constexpr int OSEG = 32;                  // chunks per carry segment
+constexpr int OCTAS = 6;                  // CTAs an SM the chunks are made for
 constexpr uint32_t EN_HERE = 0x80u;       // mark of an EN in a tile's noted statuses
+// An owner with more than HEAVY ops in a tile, and HEAVY_SLOT for each of its
+// bytes, has them walked in pieces.  Its thread alone takes about 35 cycles an op
+// while the others wait; a warp two walks of a 4th to a 32nd of that and a pass over
+// the pieces' bytes (with HEAVY alone, lists a little longer than that took 1 M
+// calls over 16,400 arrays from 2.41 to 3.31 ms, as they are walked a few at a time).
+// 16,000,000 guarded ops, 9 of 10 on one array of 1,000 / 30,000: 3.07 /
+// 6.78 ms by its thread alone, 0.45 / 1.56 so.
+constexpr int HEAVY = 128, HEAVY_SLOT = 4;
 
 // Owner of variable v among NT threads, and the offset of its byte in a row
 // without the owner's part.  v = NT h + l is owned by thread (l + 37 h) mod NT
@@ -58,11 +69,21 @@ __host__ __device__ __forceinline__ uint32_t owner_of(uint32_t v)
 {
     return (v + 37u * (v / NT)) & (NT - 1);
 }
+// Offset of an owner's h-th byte, and which one an offset is.
+template <int NT>
+__device__ __forceinline__ uint32_t addr_of_slot(uint32_t h)
+{
+    return (h >> 2) * (4 * NT) | (h & 3u);
+}
+template <int NT>
+__device__ __forceinline__ uint32_t slot_of(uint32_t addr)
+{
+    return (addr / (4 * NT)) << 2 | (addr & 3u);
+}
 template <int NT>
 __device__ __forceinline__ uint32_t addr_of(uint32_t v)
 {
-    const uint32_t h = v / NT;
-    return (h >> 2) * (4 * NT) | (h & 3u);
+    return addr_of_slot<NT>(v / NT);
 }
 template <int NT>
 __host__ __device__ __forceinline__ int64_t var_of(int64_t h, uint32_t owner)
@@ -98,6 +119,8 @@ struct OwnParams {
     int n_tiles;
     int n_chunks;
     int tiles_per_chunk;
+    int sort_room, walk_room;             // bytes after a CTA's row for the rows of pieces
+    int heavy;                            // owners with more ops of a tile are walked in pieces
     Tables tab;
 };
 
@@ -132,6 +155,107 @@ __device__ __forceinline__ void load_tables(OwnTables& S, const Tables& tab, boo
     }
 }
 
+// A heavy owner's ops, by a warp: entries [i0, i1) in pieces, a lane each, with a
+// row of the owner's bytes per piece (its h-th byte of piece k at h * pieces + k).
+template <int NO>
+struct Pieces {
+    uint8_t* rows;
+    int n, slots;                         // pieces, bytes an owner has
+    int a, b;                             // the lane's entries (none beyond the pieces)
+    __device__ __forceinline__ Pieces(uint8_t* rows_, int room, int slots_, int i0, int i1)
+        : rows(rows_), n(min(32, room / slots_)), slots(slots_)
+    {
+        const int lane = threadIdx.x & 31;
+        const int per = (i1 - i0 + n - 1) / n;
+        a = min(i0 + lane * per, i1);
+        b = lane < n ? min(a + per, i1) : a;
+    }
+    __device__ __forceinline__ uint8_t* at(uint32_t e) const
+    {
+        return rows + slot_of<NO>(ent_addr(e)) * n + (threadIdx.x & 31);
+    }
+    // a byte for all: the start of a fold
+    __device__ __forceinline__ void fill(uint32_t x)
+    {
+        __syncwarp();
+        uint32_t* w = reinterpret_cast<uint32_t*>(rows);
+        for (int i = threadIdx.x & 31; i < slots * n / 4; i += 32) w[i] = x * 0x01010101u;
+        __syncwarp();
+    }
+    // f(the row's byte of a slot, the pieces' bytes of it)
+    template <typename F>
+    __device__ __forceinline__ void each_slot(uint8_t* mine, F&& f)
+    {
+        __syncwarp();
+        for (int h = threadIdx.x & 31; h < slots; h += 32) f(mine + addr_of_slot<NO>(h), rows + h * n);
+        __syncwarp();
+    }
+};
+
+// f(owner, its pieces) for the tile's heavy owners, dealt to as many of the CTA's
+// warps as have room for eight pieces (room after the row: at least four).
+template <int NO, typename F>
+__device__ __forceinline__ void for_heavy(const OwnParams& p, const uint16_t* start, uint8_t* vec, int room, F&& f)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t m[NO / 32];
+    int K = 0;
+#pragma unroll
+    for (int w = 0; w < NO / 32; ++w) {
+        m[w] = __ballot_sync(0xffffffffu, start[32 * w + lane + 1] - start[32 * w + lane] > p.heavy);
+        K += __popc(m[w]);
+    }
+    const int slots = (int)(p.row / NO);
+    const int C = min(min(K, (int)blockDim.x / 32), max(1, room / (8 * slots)));
+    if (warp >= C) return;
+    const int share = room / C & ~15;
+    int j = 0;
+#pragma unroll
+    for (int w = 0; w < NO / 32; ++w)
+        for (uint32_t r = m[w]; r; r &= r - 1, ++j)
+            if (j % C == warp) {
+                const int o = 32 * w + __ffs(r) - 1;
+                f(o, Pieces<NO>(vec + p.row + warp * share, share, slots, start[o], start[o + 1]));
+            }
+}
+
+// The functions of the pieces composed onto the row's function.
+template <int NO>
+__device__ __forceinline__ void compose_pieces(Pieces<NO>& P, uint8_t* mine, const Tables& tab, int shift)
+{
+    P.each_slot(mine, [&](uint8_t* a, const uint8_t* q) {
+        uint32_t f = *a >> shift;
+        for (int k = 0; k < P.n; ++k)
+            if (q[k] != tab.identity) f = tab.comp[f * MAX_ELEMS + q[k]];
+        *a = (uint8_t)(f << shift | (*a & ((1u << shift) - 1u)));
+    });
+}
+// ... applied to the row's status (bits 0-2): each piece's function becomes the
+// status at its start.
+template <int NO>
+__device__ __forceinline__ void statuses_of_pieces(Pieces<NO>& P, uint8_t* mine, const Tables& tab)
+{
+    P.each_slot(mine, [&](uint8_t* a, uint8_t* q) {
+        uint32_t s = *a & 7u;
+        for (int k = 0; k < P.n; ++k) {
+            const uint32_t f = q[k];
+            q[k] = (uint8_t)s;
+            if (f != tab.identity) s = tab.app[f * 8 + s];
+        }
+        *a = (uint8_t)((*a & 0xF8u) | s);
+    });
+}
+template <int NO>
+__device__ __forceinline__ void fold_pieces(Pieces<NO>& P, const uint32_t* ent, const OwnTables& T, uint32_t identity)
+{
+    P.fill(identity);
+    for (int i = P.a; i < P.b; ++i) {
+        const uint32_t e = ent[i];
+        uint8_t* q = P.at(e);
+        *q = (uint8_t)T.then(*q, ent_code4(e));
+    }
+}
+
 // NO owners; the sort runs on NS threads, OPT ops each, the walks on NO.
 template <int NO, int NS, int OPT>
 struct SortSmem {
@@ -142,6 +266,15 @@ struct SortSmem {
     __align__(16) uint32_t ent[NS * OPT];
 };
 
+// (1) heavy owners
+template <int NO, int NS, int OPT>
+__device__ __noinline__ void sort_heavy(const OwnParams& p, SortSmem<NO, NS, OPT>& S, uint8_t* vec)
+{
+    for_heavy<NO>(p, S.start, vec, p.sort_room, [&](int o, Pieces<NO> P) {
+        fold_pieces(P, S.ent, S.T, p.tab.identity);
+        compose_pieces(P, vec + 4 * o, p.tab, 0);
+    });
+}
 // (1) sort and reduce
 template <int NO, int NS, int OPT, bool GUARDED>
 __global__ void __launch_bounds__(NS, 768 / NS) own_sort_kernel(const __grid_constant__ OwnParams p)
@@ -247,7 +380,7 @@ __global__ void __launch_bounds__(NS, 768 / NS) own_sort_kernel(const __grid_con
             }
             if (t == NO - 1) S.start[NO] = (uint16_t)n;
         }
-        __syncthreads();
+        const bool heavy = __syncthreads_or(sum > p.heavy);
 #pragma unroll
         for (int u = 0; u < OPT; ++u) {
             if (32 * u < left) {
@@ -260,11 +393,12 @@ __global__ void __launch_bounds__(NS, 768 / NS) own_sort_kernel(const __grid_con
         for (int i = 4 * t; i < n; i += 4 * NS)
             *reinterpret_cast<uint4*>(p.sorted + base + i) = *reinterpret_cast<const uint4*>(S.ent + i);
         // each owner folds its ops in order
+        if (heavy) sort_heavy<NO, NS, OPT>(p, S, vec);
         if (t < NO) {
-            const int i1 = S.start[t + 1];
+            const int i0 = S.start[t], i1 = S.start[t + 1];
             uint8_t* const mine = vec + 4 * t;
 #pragma unroll 2
-            for (int i = S.start[t]; i < i1; ++i) {
+            for (int i = i1 - i0 > p.heavy ? i1 : i0; i < i1; ++i) {
                 const uint32_t e = S.ent[i];
                 uint8_t* a = mine + ent_addr(e);
                 *a = (uint8_t)S.T.then(*a, ent_code4(e));
@@ -284,11 +418,11 @@ struct WalkSmem {
     __align__(16) uint32_t ent[TILE];
 };
 
+// The tile's entries and first entries of the owners; whether one is heavy.
 template <int NT, int TILE>
-__device__ __forceinline__ int load_tile(const OwnParams& p, WalkSmem<NT, TILE>& S, int tile)
+__device__ __forceinline__ bool load_tile(const OwnParams& p, WalkSmem<NT, TILE>& S, int tile, int n)
 {
     const int64_t base = (int64_t)tile * TILE;
-    const int n = (int)min((int64_t)TILE, p.n_ops - base);
     const int t = threadIdx.x;
     if (n == TILE) {
         uint4 q[TILE / NT / 4];
@@ -300,10 +434,101 @@ __device__ __forceinline__ int load_tile(const OwnParams& p, WalkSmem<NT, TILE>&
     } else {
         for (int i = t; i < n; i += NT) S.ent[i] = p.sorted[base + i];
     }
-    S.start[t] = p.starts[(int64_t)tile * NT + t];
+    const uint16_t* starts = p.starts + (int64_t)tile * NT;
+    const int i0 = starts[t], i1 = t < NT - 1 ? starts[t + 1] : n;
+    S.start[t] = (uint16_t)i0;
     if (t == NT - 1) S.start[NT] = (uint16_t)n;
-    __syncthreads();
-    return n;
+    return __syncthreads_or(i1 - i0 > p.heavy);
+}
+
+// Heavy owners' ops as the owners' threads do it below.  (2b) The statuses before
+// the ENs noted.
+template <int NT, int TILE>
+__device__ __noinline__ void note_heavy(const OwnParams& p, WalkSmem<NT, TILE>& S, uint8_t* vec, uint32_t nks, uint32_t nv)
+{
+    for_heavy<NT>(p, S.start, vec, p.walk_room, [&](int o, Pieces<NT> P) {
+        uint8_t* const mine = vec + 4 * o;
+        const int i0 = S.start[o], i1 = S.start[o + 1];
+        fold_pieces(P, S.ent, S.T, p.tab.identity);
+        statuses_of_pieces(P, mine, p.tab);
+        uint32_t e = P.a > i0 ? S.ent[P.a - 1] : 0u;
+        for (int i = P.a; i < P.b; ++i) {
+            const uint32_t before = e;
+            e = S.ent[i];
+            const uint32_t c4 = ent_code4(e);
+            uint8_t* q = P.at(e);
+            const uint32_t s0 = *q;
+            if ((c4 & 28u) == 4 * AMC_K_EN && e - before != (1u << POSB | 1u))
+                S.out[ent_pos(e)] = (uint8_t)(EN_HERE | (c4 & 32u) | s0);
+            *q = (uint8_t)S.T.step(s0, c4);
+        }
+        if ((threadIdx.x & 31) == 0 && (nks & 0xEFu) == AMC_K_EN && owner_of<NT>(nv) == (uint32_t)o &&
+            S.ent[i1 - 1] != (addr_of<NT>(nv) << 16 | (AMC_K_GT | ((nks >> 1) & 8u)) << POSB | (uint32_t)(TILE - 1)))
+            S.out[TILE] = (uint8_t)(EN_HERE | ((nks << 1) & 32u) | (mine[addr_of<NT>(nv)] & 7u));
+    });
+}
+// A GT whose guard finds the side invalid becomes a Pull (also in p.sorted);
+// false where no EN follows it.
+template <int NT, int TILE>
+__device__ __forceinline__ bool resolve(const OwnParams& p, const WalkSmem<NT, TILE>& S, int64_t i, uint32_t e, uint32_t& c4)
+{
+    if ((c4 & 28u) != 4 * AMC_K_GT) return true;
+    const uint32_t gs = S.out[ent_pos(e) + 1];
+    const bool pair = ((gs ^ c4 ^ EN_HERE) & (EN_HERE | 32u)) == 0;
+    // the transfer happens where the EN's variable is invalid on the side
+    // (neither flag of F is set)
+    if (pair && !(gs & ((c4 & 32u) ? 2u : 1u))) {
+        c4 ^= 4 * (AMC_K_GT ^ AMC_K_PULL);
+        p.sorted[i] = e ^ (AMC_K_GT ^ AMC_K_PULL) << POSB;
+    }
+    return pair;
+}
+// ... the resolved ops folded; false where a GT has no EN.
+template <int NT, int TILE>
+__device__ __noinline__ bool resolve_heavy(const OwnParams& p, WalkSmem<NT, TILE>& S, uint8_t* vec, int64_t base)
+{
+    bool ok = true;
+    for_heavy<NT>(p, S.start, vec, p.walk_room, [&](int o, Pieces<NT> P) {
+        P.fill(p.tab.identity);
+        for (int i = P.a; i < P.b; ++i) {
+            const uint32_t e = S.ent[i];
+            uint32_t c4 = ent_code4(e);
+            ok &= resolve(p, S, base + i, e, c4);
+            uint8_t* q = P.at(e);
+            *q = (uint8_t)S.T.then(*q, c4);
+        }
+        compose_pieces(P, vec + 4 * o, p.tab, 3);
+    });
+    return ok;
+}
+// The op's status noted; its first fault (a variable becomes stuck once).
+template <int NT, int TILE>
+__device__ __forceinline__ uint32_t apply_op(const OwnParams& p, WalkSmem<NT, TILE>& S, int64_t base, uint32_t e, int owner,
+                                             uint8_t* a, uint32_t gmin)
+{
+    const uint32_t pre = *a;
+    const uint32_t post = S.T.step(pre, ent_code4(e));
+    *a = (uint8_t)post;
+    S.out[ent_pos(e)] = (uint8_t)post;
+    if (post == ST_F && pre != ST_F) {
+        const uint32_t g = (uint32_t)base + ent_pos(e);
+        p.vff[var_of<NT>(slot_of<NT>(ent_addr(e)), owner)] = (int32_t)g;
+        gmin = min(gmin, g);
+    }
+    return gmin;
+}
+template <int NT, int TILE>
+__device__ __noinline__ uint32_t apply_heavy(const OwnParams& p, WalkSmem<NT, TILE>& S, uint8_t* vec, int64_t base, uint32_t gmin)
+{
+    for_heavy<NT>(p, S.start, vec, p.walk_room, [&](int o, Pieces<NT> P) {
+        fold_pieces(P, S.ent, S.T, p.tab.identity);
+        statuses_of_pieces(P, vec + 4 * o, p.tab);
+        for (int i = P.a; i < P.b; ++i) {
+            const uint32_t e = S.ent[i];
+            gmin = apply_op(p, S, base, e, o, P.at(e), gmin);
+        }
+    });
+    return gmin;
 }
 
 // (2b) GTs resolved and the resolved ops folded.  Row byte: the variable's
@@ -334,8 +559,9 @@ __global__ void __launch_bounds__(NT) own_resolve_kernel(const __grid_constant__
             if (nv >= (uint32_t)p.n_vars) nv = 0;
         }
         for (int i = t; i < TILE / 16 + 1; i += NT) reinterpret_cast<uint4*>(S.out)[i] = make_uint4(0, 0, 0, 0);
-        load_tile<NT, TILE>(p, S, tile);
-        const int i0 = S.start[t], i1 = S.start[t + 1];
+        const bool heavy = load_tile<NT, TILE>(p, S, tile, (int)min((int64_t)TILE, p.n_ops - base));
+        const int i1 = S.start[t + 1], i0 = i1 - S.start[t] > p.heavy ? i1 : S.start[t];
+        if (heavy) note_heavy<NT, TILE>(p, S, vec, nks, nv);
         uint32_t e = 0;
         for (int i = i0; i < i1; ++i) {
             const uint32_t before = e;
@@ -349,27 +575,18 @@ __global__ void __launch_bounds__(NT) own_resolve_kernel(const __grid_constant__
                 S.out[ent_pos(e)] = (uint8_t)(EN_HERE | (c4 & 32u) | s0);
             *a = (uint8_t)((x & 0xF8u) | S.T.step(s0, c4));
         }
-        if ((nks & 0xEFu) == AMC_K_EN && owner_of<NT>(nv) == (uint32_t)t &&
+        if ((nks & 0xEFu) == AMC_K_EN && owner_of<NT>(nv) == (uint32_t)t && i1 - S.start[t] <= p.heavy &&
             (i1 == i0 || e != (addr_of<NT>(nv) << 16 | (AMC_K_GT | ((nks >> 1) & 8u)) << POSB | (uint32_t)(TILE - 1))))
             S.out[TILE] = (uint8_t)(EN_HERE | ((nks << 1) & 32u) | (mine[addr_of<NT>(nv)] & 7u));
         __syncthreads();
         bool bad = false;
+        if (heavy) bad = !resolve_heavy<NT, TILE>(p, S, vec, base);
         for (int i = i0; i < i1; ++i) {
             e = S.ent[i];
             uint32_t c4 = ent_code4(e);
             uint8_t* a = mine + ent_addr(e);
             const uint32_t x = *a;
-            if ((c4 & 28u) == 4 * AMC_K_GT) {
-                const uint32_t gs = S.out[ent_pos(e) + 1];
-                const bool pair = ((gs ^ c4 ^ EN_HERE) & (EN_HERE | 32u)) == 0;
-                bad |= !pair;
-                // the transfer happens where the EN's variable is invalid on the side
-                // (neither flag of F is set)
-                if (pair && !(gs & ((c4 & 32u) ? 2u : 1u))) {
-                    c4 ^= 4 * (AMC_K_GT ^ AMC_K_PULL);
-                    p.sorted[base + i] = e ^ (AMC_K_GT ^ AMC_K_PULL) << POSB;
-                }
-            }
+            bad |= !resolve(p, S, base + i, e, c4);
             *a = (uint8_t)((x & 7u) | S.T.then(x >> 3, c4) << 3);
         }
         if (bad) raise_error(p.err, AMC_E_INVALID);
@@ -395,25 +612,25 @@ __global__ void __launch_bounds__(NT) own_apply_kernel(const __grid_constant__ O
     const int t0 = blockIdx.x * p.tiles_per_chunk;
     const int t1 = min(t0 + p.tiles_per_chunk, p.n_tiles);
     const bool out16 = (uintptr_t)p.step % 16 == 0;
+    bool comp = false;                                     // the composition table is loaded
     uint32_t gmin = 0xFFFFFFFFu;
     for (int tile = t0; tile < t1; ++tile) {
         const int64_t base = (int64_t)tile * TILE;
-        const int n = load_tile<NT, TILE>(p, S, tile);
-        const int i1 = S.start[t + 1];
-#pragma unroll 2
-        for (int i = S.start[t]; i < i1; ++i) {
-            const uint32_t e = S.ent[i];
-            uint8_t* a = mine + ent_addr(e);
-            const uint32_t pre = *a;
-            const uint32_t post = S.T.step(pre, ent_code4(e));
-            *a = (uint8_t)post;
-            S.out[ent_pos(e)] = (uint8_t)post;
-            if (post == ST_F && pre != ST_F) {             // a variable becomes stuck once
-                const uint32_t g = (uint32_t)base + ent_pos(e);
-                const uint32_t h = (ent_addr(e) / (4 * NT)) << 2 | (ent_addr(e) & 3u);
-                p.vff[var_of<NT>(h, t)] = (int32_t)g;
-                gmin = min(gmin, g);
+        const int n = (int)min((int64_t)TILE, p.n_ops - base);
+        const bool heavy = load_tile<NT, TILE>(p, S, tile, n);
+        const int i0 = S.start[t], i1 = S.start[t + 1];
+        if (heavy) {
+            if (!comp) {
+                load_tables(S.T, p.tab, true);
+                __syncthreads();
+                comp = true;
             }
+            gmin = apply_heavy<NT, TILE>(p, S, vec, base, gmin);
+        }
+#pragma unroll 2
+        for (int i = i1 - i0 > p.heavy ? i1 : i0; i < i1; ++i) {
+            const uint32_t e = S.ent[i];
+            gmin = apply_op(p, S, base, e, t, mine + ent_addr(e), gmin);
         }
         __syncthreads();
         if (out16 && n == TILE) {
@@ -573,7 +790,7 @@ OwnShape shape_of(int64_t n_ops, int32_t n_vars, bool wide)
     S.no = wide ? 256 : 128;
     const int64_t h = ((int64_t)n_vars + S.no - 1) / S.no;
     S.row = (h + 3) / 4 * 4 * S.no;
-    const int want = 152 * 6;
+    const int want = 152 * OCTAS;
     S.tile = wide || n_ops >= (int64_t)want * 4096 ? 4096 : 1024;
     S.n_tiles = (int)((n_ops + S.tile - 1) / S.tile);
     const int c = S.n_tiles < want ? S.n_tiles : want;
@@ -628,17 +845,34 @@ int run_carry(OwnParams p, const OwnShape& S, bool one_carry, bool last, cudaStr
     return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
 }
 
+// Room for the rows of pieces, of CTAs that need `bytes` without it: what does not
+// cost an SM one of its (at most `ctas`) CTAs, at least four pieces.
+constexpr int ROOM_MAX = 8192;
+int room_for(int owners, size_t row, size_t bytes, int ctas)
+{
+    constexpr size_t SM = 228 << 10, EACH = 1024;          // shared memory; kept by the system per CTA
+    const size_t fit = SM / (bytes + EACH);
+    if (fit < (size_t)ctas) ctas = fit > 0 ? (int)fit : 1;
+    const int64_t left = ((int64_t)(SM / ctas) - (int64_t)(bytes + EACH)) / 16 * 16;
+    const int64_t least = (int64_t)align_up(4 * (row / owners), 16);
+    return (int)(left < least ? least : left < ROOM_MAX ? left : ROOM_MAX);
+}
+
 template <int NO, int NS, int OPT>
 int run_owner(const ScanLaunch& L, const OwnShape& S, bool guarded, bool one_carry, uint8_t* ws, cudaStream_t s)
 {
     constexpr int TILE = NS * OPT;
-    const OwnParams p = params_of(L, S, ws);
-    const size_t smS = sizeof(SortSmem<NO, NS, OPT>) + (size_t)S.row;
-    const size_t smW = sizeof(WalkSmem<NO, TILE>) + (size_t)S.row;
+    OwnParams p = params_of(L, S, ws);
+    const size_t row = (size_t)S.row;
+    p.heavy = HEAVY + HEAVY_SLOT * (int)(row / NO);
+    p.sort_room = room_for(NO, row, sizeof(SortSmem<NO, NS, OPT>) + row, 768 / NS);
+    p.walk_room = room_for(NO, row, sizeof(WalkSmem<NO, TILE>) + row, OCTAS);
+    const size_t smS = sizeof(SortSmem<NO, NS, OPT>) + row + p.sort_room;
+    const size_t smW = sizeof(WalkSmem<NO, TILE>) + row + p.walk_room;
     auto sort = guarded ? own_sort_kernel<NO, NS, OPT, true> : own_sort_kernel<NO, NS, OPT, false>;
-    const size_t row = NO == 128 ? OWN_NARROW_VARS : OWN_MAX_VARS;       // the longest
-    const size_t mS = sizeof(SortSmem<NO, NS, OPT>) + row, mW = sizeof(WalkSmem<NO, TILE>) + row;
-    if (smS > mS || !allow_smem<own_sort_kernel<NO, NS, OPT, true>>(mS) ||
+    const size_t most = (NO == 128 ? OWN_NARROW_VARS : OWN_MAX_VARS) + ROOM_MAX;     // of row and room
+    const size_t mS = sizeof(SortSmem<NO, NS, OPT>) + most, mW = sizeof(WalkSmem<NO, TILE>) + most;
+    if (smS > mS || smW > mW || !allow_smem<own_sort_kernel<NO, NS, OPT, true>>(mS) ||
         !allow_smem<own_sort_kernel<NO, NS, OPT, false>>(mS) || !allow_smem<own_apply_kernel<NO, TILE>>(mW) ||
         !allow_smem<own_resolve_kernel<NO, TILE>>(mW))
         return AMC_E_CUDA;
