@@ -134,10 +134,10 @@ __device__ void run_unit(const BatchParams& p, const Unit& u, WarpSmem& S, const
     // token of the segment in the warp's own rows (the five passes of a
     // segment run at once on different warps)
     auto save_at = [&](int d, int64_t q) -> uint8_t* {
-        return apply ? p.save + (int64_t)d * p.n_tokens + q : u.rsave + (int64_t)d * seg_max_of(p.split) + (q - t0);
+        return apply ? p.save + p.save_rows * t0 + d * (t1 - t0) + (q - t0) : u.rsave + (int64_t)d * seg_max_of(p.split) + (q - t0);
     };
     auto alt_at = [&](int d, int64_t q) -> uint8_t* {
-        return apply ? p.alt + (int64_t)d * p.n_tokens + q : u.ralt + (int64_t)d * seg_max_of(p.split) + (q - t0);
+        return apply ? p.alt + p.save_rows * t0 + d * (t1 - t0) + (q - t0) : u.ralt + (int64_t)d * seg_max_of(p.split) + (q - t0);
     };
     auto range_end = [&]() -> int64_t { return depth ? fpos[(depth - 1) * 3 + 2] : t1; };
     // parallel helper over the op tokens of (a, b)
@@ -364,6 +364,7 @@ __global__ void __launch_bounds__(BWARPS * 32, MINB) batch_kernel(const BatchPar
 {
     __shared__ WarpSmem smem[BWARPS];
     __shared__ TabSmem tab;
+    cudaTriggerProgrammaticLaunchCompletion();             // (the evaluation by variables starts beside this)
     if (gated_off(pl.gate)) return;
     const int w = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -842,10 +843,6 @@ int launch_batch(const BatchLaunch& B, cudaStream_t s)
             order_units_kernel<<<1, 1024, 0, s>>>(order, pl.unit_off, B.n_progs, pl.ord_off, pl.gate);
         p.order = order;
     }
-    if (by_vars) {
-        const int rc = launch_batch_vars(p, B.max_ctas, vars_queue, gate + 1, s);
-        if (rc) return rc;
-    }
     if (!pl.simple) {
         const int64_t rgrid = grid < L.red_ctas ? grid : L.red_ctas;
         if (rgrid > 0) kern<<<(unsigned)rgrid, BWARPS * 32, 0, s>>>(p, pl, 0);      // reduce
@@ -853,6 +850,13 @@ int launch_batch(const BatchLaunch& B, cudaStream_t s)
         if (cudaMemsetAsync(p.queue_head, 0, 8, s) != cudaSuccess) return AMC_E_CUDA;
     }
     kern<<<(unsigned)grid, BWARPS * 32, 0, s>>>(p, pl, 1);       // apply
+    if (by_vars) {
+        // beside the apply kernel, whose longest program may take as long as all of
+        // these: 64 programs of 60,000 tokens, some of them left to it, 40.8 ms one after
+        // the other, 33.4 so
+        const int rc = launch_batch_vars(p, B.max_ctas, vars_queue, gate + 1, s);
+        if (rc) return rc;
+    }
     if (B.profile & 2) profile_end(s);
     return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
 }

@@ -17,8 +17,8 @@ struct BatchParams {
     uint8_t* step_mask;
     uint8_t* final_mask;
     int64_t* prog_first_fault;
-    uint8_t* save;                 // [AMC_MAX_DEPTH][n_tokens]
-    uint8_t* alt;                  // [AMC_MAX_DEPTH][n_tokens]
+    uint8_t* save;                 // [n_tokens][save_rows]: a unit of tokens [a, b) has the bytes from
+    uint8_t* alt;                  //   save_rows a to save_rows b, rows of b - a in them
     const int32_t* order;          // nullable: program queue order
     uint64_t* queue_head;
     int* err;
@@ -71,7 +71,8 @@ __device__ __forceinline__ bool program_by_vars(const BatchParams& p, int64_t pr
     return program_fits_vars(b - a, nv, p.split);
 }
 // Those programs of the batch (p.save / p.alt with AMC_MAX_DEPTH rows: 8 bytes
-// a token each); *queue is zero.  None when *off (device) is set.
+// a token each); *queue is zero.  None when *off (device) is set.  Starts beside the
+// kernel launched before it, from all before which it takes its input.
 int launch_batch_vars(const BatchParams& p, int64_t max_ctas, unsigned long long* queue, const int* off, cudaStream_t s);
 
 size_t batch_workspace_bytes(int64_t n_tokens, int64_t n_progs);

@@ -86,11 +86,12 @@ __device__ void run_program(const BatchParams& p, int64_t prog, VarSmem& S, uint
     const uint8_t* init = p.init_mask ? p.init_mask + v0 : nullptr;
     constexpr uint32_t VI = 1u << AMC_ST_VI;
     // words of the ops, the constructs opened before them, chains (first op | its
-    // variable << 16), constructs (at most one per two tokens)
-    uint32_t* W = reinterpret_cast<uint32_t*>(p.save) + t0;
-    uint16_t* opened = reinterpret_cast<uint16_t*>(p.alt) + t0;
-    uint32_t* heads = reinterpret_cast<uint32_t*>(p.save) + p.n_tokens + t0;
-    uint64_t* C = reinterpret_cast<uint64_t*>(p.alt + (2 * p.n_tokens + 7) / 8 * 8) + (t0 + 1) / 2;
+    // variable << 16), constructs (at most one per two tokens): 8 and at most 8
+    // bytes per token of the program's own (the kernel beside this has the others')
+    uint32_t* W = reinterpret_cast<uint32_t*>(p.save + 8 * t0);
+    uint16_t* opened = reinterpret_cast<uint16_t*>(p.alt + 8 * t0);
+    uint32_t* heads = W + len;
+    uint64_t* C = reinterpret_cast<uint64_t*>(p.alt + 8 * t0) + (len + 3) / 4;
     for (int v = lane; v < (nv + 1) / 2; v += 32) reinterpret_cast<uint32_t*>(tail)[v] = ~0u;
     // variables without an op keep their set
     for (int v = lane; v < nv; v += 32) fin[v] = init ? init[v] : (uint8_t)VI;
@@ -352,14 +353,13 @@ __device__ void run_program(const BatchParams& p, int64_t prog, VarSmem& S, uint
 __global__ void __launch_bounds__(VWARPS * 32, VCTAS) vars_kernel(const __grid_constant__ BatchParams p,
                                                              unsigned long long* queue, const int* off)
 {
-    if (*off) return;
     extern __shared__ __align__(16) uint8_t smem[];
     VarSmem& S = *reinterpret_cast<VarSmem*>(smem);
     for (int i = threadIdx.x; i < 16 * 32; i += blockDim.x) S.img[i] = p.tab.img[i];
     if (threadIdx.x < 16) S.flt[threadIdx.x] = p.tab.flt[threadIdx.x];
     __syncthreads();
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (;;) {
+    while (!*off) {
         long long i = 0;
         if (lane == 0) i = (long long)atomicAdd(queue, 1ull);
         i = __shfl_sync(0xffffffffu, i, 0);
@@ -369,6 +369,8 @@ __global__ void __launch_bounds__(VWARPS * 32, VCTAS) vars_kernel(const __grid_c
         run_program(p, prog, S, S.tail[w]);
         __syncwarp();
     }
+    // this kernel ends no earlier than the one it started beside
+    cudaGridDependencySynchronize();
 }
 
 }  // namespace
@@ -383,7 +385,7 @@ int launch_batch_vars(const BatchParams& p, int64_t max_ctas, unsigned long long
     const int64_t need = (p.n_progs + VWARPS - 1) / VWARPS;
     if (grid > need) grid = need;
     if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
-    vars_kernel<<<(unsigned)grid, VWARPS * 32, sizeof(VarSmem), s>>>(p, queue, off);
+    chain(vars_kernel, (unsigned)grid, VWARPS * 32, sizeof(VarSmem), s)(p, queue, off);
     return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
 }
 
