@@ -53,3 +53,12 @@ def test_long_programs_beside(amc, oracle_mod):
     # more than 65,535 tokens: cut into segments
     check(amc, oracle_mod, parts(dict(n_progs=5, seed=23, median=70000.0, sigma=0.1, vars_lo=3, vars_hi=200),
                                  dict(n_progs=400, seed=24, median=700.0, vars_lo=1, vars_hi=300, **DEEP)))
+
+
+@pytest.mark.parametrize("nv", [1, 2, 33])
+@pytest.mark.parametrize("p_if,p_while", [(0.0, 0.0), (0.004, 0.0), (0.002, 0.002), (0.02, 0.01)])
+def test_few_constructs(amc, oracle_mod, nv, p_if, p_while):
+    # stretches of ops in no construct, none to several hundred ops long
+    progs = parts(dict(n_progs=200, seed=25, median=900.0, vars_lo=nv, vars_hi=nv, p_if=p_if, p_while=p_while),
+                  dict(n_progs=40, seed=26, median=31.0, sigma=0.2, vars_lo=nv, vars_hi=nv, p_if=0.0, p_while=0.0))
+    check(amc, oracle_mod, progs)
