@@ -576,25 +576,8 @@ int amc_check_batch(const uint8_t* tok_kind_side, const int32_t* tok_payload, co
     B.workspace = workspace;
     B.profile = 3;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // candidates (longest-first queue): registers fitted to six or four CTAs
-    // per SM
-    auto shape = [&](BatchLaunch X, int i) {
-        X.longest_first = 1;
-        X.regs_capped = (i & 1) ? 0 : 1;
-        return X;
-    };
-    const std::string key = shape_key("batch", n_tokens, n_progs, 0);
-    if (!graph_capture || s == nullptr)
-        return autotune_run(key, 2, 0, s, [&](int i) { return launch_batch(shape(B, i), s); });
-    {
-        // tune outside the capture first (no-op when the key is cached)
-        const int rc0 = autotune_lookup(key) >= 0
-                            ? AMC_OK
-                            : autotune_run(key, 2, 0, s, [&](int i) { return launch_batch(shape(B, i), s); });
-        if (rc0) return rc0;
-        const int pick = autotune_lookup(key);
-        B = shape(B, pick >= 0 ? pick : 0);
-    }
+    B.longest_first = 1;
+    if (!graph_capture || s == nullptr) return launch_batch(B, s);
     int dev = 0;
     cudaGetDevice(&dev);
     std::vector<uintptr_t> gkey = {(uintptr_t)dev,          (uintptr_t)s,           (uintptr_t)tok_kind_side,

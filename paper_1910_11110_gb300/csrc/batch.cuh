@@ -43,7 +43,6 @@ struct BatchLaunch {
     void* workspace = nullptr;
     int longest_first = 1;
     int max_ctas = 0;
-    int regs_capped = 1;           // registers fitted to 6 CTAs per SM (else to 4)
     int no_split = 0;              // never split a program (no reduce-pass scratch)
     int save_rows = AMC_MAX_DEPTH; // construct levels with save / alt rows (0: straight-line only)
     int profile = 0;
