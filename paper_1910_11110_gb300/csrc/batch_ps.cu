@@ -76,7 +76,9 @@ struct PsTab {
 
 constexpr int PS_SMALL_VARS = 256;
 constexpr int PS_SHARE = PS_SMALL_VARS / 32;      // warps on a long program
-constexpr int64_t PS_LONG = 2048;                 // tokens of the shortest one
+// tokens of the shortest one (one program of 1,024 to 2,047, over its guard alone: 725 us
+// by one warp with its state in shared memory, 567 so; over 17 variables 342 and 261)
+constexpr int64_t PS_LONG = 1024;
 
 constexpr int PS_ROWS = 4;                        // construct levels whose rows lie in shared memory
 
