@@ -64,7 +64,7 @@ __device__ __forceinline__ uint32_t seg_combine(uint32_t x, uint32_t y, const ui
 }
 
 // Thread loads of a tile's keys / values in blocked arrangement (thread t:
-// pairs [16 t, 16 t + 16) of the tile); pairs past m are left as NOKEY.
+// pairs [SE t, SE t + SE) of the tile); pairs past m are left as NOKEY.
 __device__ __forceinline__ void load_blocked(const uint32_t* __restrict__ a, int64_t b, int m, uint32_t (&x)[SE],
                                              uint32_t fill)
 {
@@ -316,7 +316,7 @@ struct SegParams {
 
 constexpr uint32_t TS_VAL = 0x1FFu;      // a scan value: element (bits 0-4), "a run starts inside" (bit 8)
 
-// Per thread: its 16 sorted pairs, run starts and the fold of its pairs.
+// Per thread: its SE sorted pairs, run starts and the fold of its pairs.
 struct ThreadRun {
     uint32_t k[SE], v[SE];
     uint32_t heads;             // bit u: pair u starts a variable's run

@@ -1764,7 +1764,7 @@ int scan_trace_plan(const ScanLaunch& L, int* launches)
                ((L.dense == 1 && dense_forced_ok(L.n_ops, L.n_vars)) || scan_dense_eligible(L.n_ops, L.n_vars))) {
         const char* e = getenv("AMC_SCAN_DENSE_SORT");
         const bool warp = L.n_vars <= 8192 && !(e && e[0] == '1');
-        n = warp ? 5 : 3;                                   // chunk, reduce, carry, expand, chunk; or reduce, carry, apply
+        n = warp ? 5 : 3;                                   // sort, three of the carry, apply; or sort, carry, apply
         path = warp ? AMC_PATH_WARP_DENSE : AMC_PATH_DENSE;
     } else if (L.dense != 0 && (L.prefix_log2 > 0 ? scan_forced_prefix(L)
                                                   : plain && scan_prefix_eligible(L.n_ops, L.n_vars, L.init != nullptr))) {
