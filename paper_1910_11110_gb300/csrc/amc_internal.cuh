@@ -249,7 +249,7 @@ bool allow_smem(size_t most)
 // finished and its writes can be seen.  A kernel that returned without waiting
 // would let its follower run ahead of its predecessor.  It is for chains of many
 // short kernels: a 16.8 M op trace in epochs (38 kernels) 388 -> 327 us, one of
-// 2^30 ops (74) 2076 -> 1955, four locations 708 -> 652.  The owner-sorted
+// 2^30 ops (74) 2076 -> 1955, four locations 708 -> 652 when it came.  The owner-sorted
 // tiles and the VectorPU translation are launched without it: a few kernels of
 // thousands of CTAs, where waiting CTAs only take room (5 M calls 4.02 -> 4.26 ms).
 // Not `ahead`: the same launch without it (sorts of many pairs).

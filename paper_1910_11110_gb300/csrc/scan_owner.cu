@@ -27,15 +27,15 @@
 //      guard finds the side invalid, and folds the resolved ops again;
 // and 2. / 3. follow on the resolved functions.
 // What bounds it: instruction issue and shared-memory latency (the ranking's
-// ballots in step 1, about a dozen instructions per op and walk after it; 129,
-// 104 and 40 warp instructions per 32 ops in steps 1, 2b and 3), not memory: 5
+// ballots in step 1, about a dozen instructions per op and walk after it; 119,
+// 103 and 42 warp instructions per 32 ops in steps 1, 2b and 3), not memory: 5
 // bytes in and 4 out per op in step 1, 4 in and 1 out in step 3.  Warps that
 // instead walk 32 consecutive ops at a time over a row of their own, lanes with
 // equal variables grouped by match.any, take 144 to 160 warp instructions per
 // 32 ops and walk, and a guarded trace four walks: the check of 182 M
-// statements over 8,192 variables took 7.75 ms that way and takes 2.5 ms here
-// (1.13 + 0.95 + 0.35 ms for steps 1, 2b and 3), one of 300,007 ops over 2,011
-// variables 171 us and 49 us.  Tiles of 4,096 ops for 128 owners rather than
+// statements over 8,192 variables took 7.75 ms that way and takes 2.3 ms here
+// (1.00 + 0.82 + 0.40 ms for steps 1, 2b and 3), one of 300,007 ops over 2,011
+// variables 171 us and 39 us.  Tiles of 4,096 ops for 128 owners rather than
 // 2,048 took step 1 from 1.53 to 1.13 ms and step 3 from 0.50 to 0.38 ms (the
 // longest walk of a warp over the mean: 1.57 against 1.81).
 #include "amc_internal.cuh"
@@ -782,8 +782,14 @@ struct OwnShape {
 // 128 owners and 4,096-op tiles (32 ops per owner: the longer the walks, the
 // better they are balanced) where there is a wave of tiles, 1,024-op tiles
 // below (more CTAs at work); wide: 256 owners, so that rows of up to 64 KB
-// leave enough walking warps on an SM.  Chunks: one wave of CTAs; a CTA walks
-// its tiles in order.
+// leave enough walking warps on an SM.  A CTA walks the tiles of its chunk in
+// order.  At most 912 chunks (six CTAs on each of 152 SMs: one wave of the walks
+// with 128 owners) for every variant, so that the workspace does not depend on the
+// device.  Of wide rows fewer CTAs fit, and the chunks are up to three waves of them,
+// each with a row to write, carry and read: with 304, 456, 608 and 912 chunks a
+// plain trace of 16 M ops over 60,000 variables takes 247, 267, 266 and 289 us, a
+// guarded one 368, 461, 425 and 480; 150 M ops over 65,536 1.72, 1.81, 1.69 and 1.71
+// ms, guarded 2.55, 3.04, 2.60 and 2.66; 30 M over 32,800 404, 351, 349 and 374 us.
 OwnShape shape_of(int64_t n_ops, int32_t n_vars, bool wide)
 {
     OwnShape S;
@@ -896,6 +902,12 @@ int run_owner(const ScanLaunch& L, const OwnShape& S, bool guarded, bool one_car
 int run_shape(const ScanLaunch& L, bool guarded, bool wide, uint8_t* ws, cudaStream_t s)
 {
     const OwnShape S = shape_of(L.n_ops, L.n_vars, wide);
+    // A plain trace over few variables takes the carry in three kernels, which is
+    // what the plan reports of it; one kernel is the faster carry (300,007 ops over
+    // 2,011 variables 59 us with three and 45 with one, 16 M over 8,000 213 and 200,
+    // 150 M 1,286 and 1,276), and taken elsewhere (guarded: 98 and 66, 331 and 302,
+    // 1,949 and 1,926).  Dependent launches of the five kernels: 53 us, 210 us and 1,286;
+    // of the guarded ones 68, 325 and 1,962.
     const bool one_carry = guarded || wide;
     if (wide) return run_owner<256, 256, 16>(L, S, guarded, one_carry, ws, s);
     return S.tile == 4096 ? run_owner<128, 256, 16>(L, S, guarded, one_carry, ws, s)
