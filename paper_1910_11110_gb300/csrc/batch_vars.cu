@@ -404,12 +404,20 @@ int launch_batch_vars(const BatchParams& p, int64_t max_ctas, unsigned long long
     int dev = 0, n_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (!allow_smem<vars_kernel>(sizeof(VarSmem))) return AMC_E_CUDA;
     int64_t grid = VCTAS * (int64_t)n_sm;
     const int64_t need = (p.n_progs + VWARPS - 1) / VWARPS;
     if (grid > need) grid = need;
     if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
-    chain(vars_kernel, (unsigned)grid, VWARPS * 32, sizeof(VarSmem), s)(p, queue, off);
+    // Few CTAs are spread over the SMs: those of the kernel before leave some SMs
+    // first, which would take all of these (40 programs of 46,000 tokens beside 40 over
+    // 4,097 and more variables: 10.7 ms with 20 CTAs on four SMs, 7.6 so).
+    // With more shared memory than it needs no SM takes more than its part, and the
+    // rest of it holds the CTAs of that kernel (18 KB each).
+    constexpr size_t SM = 228 << 10;
+    const size_t part = (size_t)((grid + n_sm - 1) / n_sm), most = SM / 2;
+    const size_t smem = part < VCTAS ? SM / (part + 1) / 16 * 16 : sizeof(VarSmem);
+    if (!allow_smem<vars_kernel>(most)) return AMC_E_CUDA;
+    chain(vars_kernel, (unsigned)grid, VWARPS * 32, smem > sizeof(VarSmem) ? smem : sizeof(VarSmem), s)(p, queue, off);
     return cudaGetLastError() == cudaSuccess ? AMC_OK : AMC_E_CUDA;
 }
 
