@@ -52,11 +52,13 @@ constexpr uint32_t EN_HERE = 0x80u;       // mark of an EN in a tile's noted sta
 // An owner with more than HEAVY ops in a tile, and HEAVY_SLOT for each of its
 // bytes, has them walked in pieces.  Its thread alone takes about 35 cycles an op
 // while the others wait; a warp two walks of a 4th to a 32nd of that and a pass over
-// the pieces' bytes (with HEAVY alone, lists a little longer than that took 1 M
-// calls over 16,400 arrays from 2.41 to 3.31 ms, as they are walked a few at a time).
-// 16,000,000 guarded ops, 9 of 10 on one array of 1,000 / 30,000: 3.07 /
+// the pieces' bytes, a few owners at a time.  From 128 ops on, tiles with many lists a
+// little longer lose: 16 M ops over 20 variables 366 us against 341 without pieces and
+// 331 so, and with no allowance for the bytes 1 M calls over 16,400 arrays 3.31 ms
+// against 2.41; 10 M ops over 8,000 Zipf ids take 304 us from 128 on, 325 so, 372 from
+// 384 on or without.  16,000,000 guarded ops, 9 of 10 on one array of 1,000 / 30,000: 3.07 /
 // 6.78 ms by its thread alone, 0.45 / 1.56 so.
-constexpr int HEAVY = 128, HEAVY_SLOT = 4;
+constexpr int HEAVY = 256, HEAVY_SLOT = 4;
 
 // Owner of variable v among NT threads, and the offset of its byte in a row
 // without the owner's part.  v = NT h + l is owned by thread (l + 37 h) mod NT
@@ -266,7 +268,7 @@ struct SortSmem {
     __align__(16) uint32_t ent[NS * OPT];
 };
 
-// (1) heavy owners
+// (1) a tile with heavy owners, the walks of the others included
 template <int NO, int NS, int OPT>
 __device__ __noinline__ void sort_heavy(const OwnParams& p, SortSmem<NO, NS, OPT>& S, uint8_t* vec)
 {
@@ -274,6 +276,14 @@ __device__ __noinline__ void sort_heavy(const OwnParams& p, SortSmem<NO, NS, OPT
         fold_pieces(P, S.ent, S.T, p.tab.identity);
         compose_pieces(P, vec + 4 * o, p.tab, 0);
     });
+    const int t = threadIdx.x;
+    if (t >= NO) return;
+    const int i1 = S.start[t + 1];
+    for (int i = i1 - S.start[t] > p.heavy ? i1 : S.start[t]; i < i1; ++i) {
+        const uint32_t e = S.ent[i];
+        uint8_t* a = vec + 4 * t + ent_addr(e);
+        *a = (uint8_t)S.T.then(*a, ent_code4(e));
+    }
 }
 // (1) sort and reduce
 template <int NO, int NS, int OPT, bool GUARDED>
@@ -393,17 +403,17 @@ __global__ void __launch_bounds__(NS, 768 / NS) own_sort_kernel(const __grid_con
         for (int i = 4 * t; i < n; i += 4 * NS)
             *reinterpret_cast<uint4*>(p.sorted + base + i) = *reinterpret_cast<const uint4*>(S.ent + i);
         // each owner folds its ops in order
-        if (heavy) sort_heavy<NO, NS, OPT>(p, S, vec);
-        if (t < NO) {
-            const int i0 = S.start[t], i1 = S.start[t + 1];
+        if (t < NO && !heavy) {
+            const int i1 = S.start[t + 1];
             uint8_t* const mine = vec + 4 * t;
 #pragma unroll 2
-            for (int i = i1 - i0 > p.heavy ? i1 : i0; i < i1; ++i) {
+            for (int i = S.start[t]; i < i1; ++i) {
                 const uint32_t e = S.ent[i];
                 uint8_t* a = mine + ent_addr(e);
                 *a = (uint8_t)S.T.then(*a, ent_code4(e));
             }
         }
+        if (heavy) sort_heavy<NO, NS, OPT>(p, S, vec);
         __syncthreads();
     }
     for (int64_t i = 16 * t; i < p.row; i += 16 * NS)
@@ -528,6 +538,11 @@ __device__ __noinline__ uint32_t apply_heavy(const OwnParams& p, WalkSmem<NT, TI
             gmin = apply_op(p, S, base, e, o, P.at(e), gmin);
         }
     });
+    const int t = threadIdx.x, i1 = S.start[t + 1];
+    for (int i = i1 - S.start[t] > p.heavy ? i1 : S.start[t]; i < i1; ++i) {
+        const uint32_t e = S.ent[i];
+        gmin = apply_op(p, S, base, e, t, vec + 4 * t + ent_addr(e), gmin);
+    }
     return gmin;
 }
 
@@ -618,19 +633,20 @@ __global__ void __launch_bounds__(NT) own_apply_kernel(const __grid_constant__ O
         const int64_t base = (int64_t)tile * TILE;
         const int n = (int)min((int64_t)TILE, p.n_ops - base);
         const bool heavy = load_tile<NT, TILE>(p, S, tile, n);
-        const int i0 = S.start[t], i1 = S.start[t + 1];
-        if (heavy) {
+        if (!heavy) {
+            const int i1 = S.start[t + 1];
+#pragma unroll 2
+            for (int i = S.start[t]; i < i1; ++i) {
+                const uint32_t e = S.ent[i];
+                gmin = apply_op(p, S, base, e, t, mine + ent_addr(e), gmin);
+            }
+        } else {
             if (!comp) {
                 load_tables(S.T, p.tab, true);
                 __syncthreads();
                 comp = true;
             }
             gmin = apply_heavy<NT, TILE>(p, S, vec, base, gmin);
-        }
-#pragma unroll 2
-        for (int i = i1 - i0 > p.heavy ? i1 : i0; i < i1; ++i) {
-            const uint32_t e = S.ent[i];
-            gmin = apply_op(p, S, base, e, t, mine + ent_addr(e), gmin);
         }
         __syncthreads();
         if (out16 && n == TILE) {

@@ -57,11 +57,11 @@ def test_hot_variables(amc, oracle_mod, monkeypatch, n, n_vars, hot, share, wide
 @pytest.mark.parametrize("n_vars", [128, 5000])
 def test_list_lengths(amc, oracle_mod, monkeypatch, more, n_vars, wide):
     # the variables of one owner have `length` ops in the tile, the others few; lists
-    # of more than 128 and 4 for each of an owner's bytes are walked in pieces
+    # of more than 256 and 4 for each of an owner's bytes are walked in pieces
     monkeypatch.setenv("AMC_TRACE_CANDIDATE", "4")
     monkeypatch.setenv("AMC_SCAN_DENSE_SORT", wide)
     no = 256 if wide == "1" else 128
-    length = 128 + 4 * (-(-n_vars // (4 * no)) * 4) + more
+    length = 256 + 4 * (-(-n_vars // (4 * no)) * 4) + more
     rng = np.random.default_rng(length)
     v = np.arange(n_vars)
     owner = (v + 37 * (v // no)) % no
